@@ -59,7 +59,7 @@ __device__ __forceinline__ void texel_coord(float x, int size, int &t, float &f)
     texel_of(__fmul_rn(x, (float)size), size, t, f);
 }
 
-// Listing 3 along one axis, both directions.  A texel of the walk continues
+// Listing 3, the four walks of an edge fragment.  A texel of a walk continues
 // the edge when it keeps the fragment's shadow-test result and shares a
 // discontinuity direction with the fragment.  Along x only the +-y
 // directions can be shared: the walk's texel has the same result as the
@@ -68,215 +68,109 @@ __device__ __forceinline__ void texel_coord(float x, int size, int &t, float &f)
 // step ends the walk).  Both facts hold with clamp-to-edge addressing too;
 // along y the same holds with the axes swapped.  A walk returns +k for an
 // end found at step k, -k for a texel that left the edge, -(max_dist+1) when
-// all steps continued: rn for the walk towards lower indices, rp for the
-// walk towards higher ones.
+// all steps continued.
 //
-// The walks read three fixed lines of the map (the row or column of the
-// fragment and its two neighbours).  `line` points at the first texel of
-// the fragment's own line, `stride` is the distance between consecutive
-// texels of a line, `pos`/`last` the fragment's index and the last index
-// along it; each direction steps a pointer along the line and holds it at
-// the border (clamp to edge).  The side lines that share a direction
-// (use_a/use_b) lie da and db elements from the line; with kAdjacent (the
-// walks along y) they are the columns i-1 and i+1, read at the immediate
-// offsets -1 and +1.  A side is only read when the fragment has a
-// discontinuity towards it, and at the map border the clamped neighbour is
-// the texel itself and shows none, so a side that is read exists and the
-// offsets never leave the map.  The two directions advance together and
-// every load of a step (of both walks; a finished walk issues none) is in
-// flight before the first test, so a step costs one memory latency.  Loads
-// of later steps are not issued ahead: the extra, mostly wasted, requests
-// cost more than the latency they hide.
-template <bool kAdjacent>
-__device__ __forceinline__ void walk_pair(const float *line, long long da, long long db, long long stride,
-                                          int pos, int last, bool use_a, bool use_b, float pz, int s0,
-                                          int max_dist, int &rn, int &rp)
+// The fragment's own discontinuities settle every walk but two at most.  A
+// walk in a direction with a discontinuity ends at its first texel (+1); one
+// along an axis without a discontinuity across it leaves the edge there
+// (-1).  Of the directions left, a straight edge keeps the two along it, a
+// corner one on each axis, a dead end one, and a texel on its own none.  So a
+// lane has two walks, A and B, each with its own step and side, and a drain
+// round of 32 fragments runs one loop as long as its longest walk, whatever
+// axes its lanes walk along (one loop per axis made a round as long as its
+// longest x walk and its longest y walk together).
+//
+// A walk reads its own line and the side line that shares the direction, at
+// a fixed offset from it (both side lines where both are in use, a thin
+// feature: the second one in a branch that most rounds skip).  A side is only read
+// when the fragment has a discontinuity towards it, and at the map border
+// the clamped neighbour is the texel itself and shows none, so a side that
+// is read exists.  A walk that reaches the border stays on its texel (clamp
+// to edge), which continues the edge, for the steps that are left: it finds
+// no end, so it is stopped there.  The loads of a step, of both walks, are in
+// flight before the first test.  Loads of later steps are not issued ahead: the extra, mostly wasted,
+// requests cost more than the latency they hide (two steps per iteration
+// with their loads together: 67.2 against 60.7 us on one 3840x2160 frame).
+//
+// Bound: the latency of the steps and the issue slots of a round's longest
+// walk.  rsmss_filter, 3840x2160 fragments on a 4096^2 map, 5 % of them on
+// edges: 76.2 us with one loop per axis, 60.7 us with this one (41 us
+// without any walk); 64 jobs of cascades in one launch: 504 against 433 us.
+// Measured against it, the same answers: the warp taking the open walks of a
+// round one pair at a time, 16 steps of each across its lanes (two ballots
+// settle a pair): 76 us when at most 8 walks are left open, 97 at 16; and
+// texture gathers, two steps each: 63.6 us, and 525 on the cascades.
+struct EdgeWalk {
+    const float *p;                // the texel reached
+    long long step, side;          // to the next texel, and to the side line's texel
+    int last;                      // the last step to take; 0 = the walk is done
+};
+
+__device__ __forceinline__ EdgeWalk edge_walk(const MapDev &m, const float *p, int i, int j, unsigned d, unsigned d4,
+                                              int max_dist)
 {
-    rn = 0;
-    rp = 0;
-    const float *pn = line + (long long)pos * stride;
-    const float *pp = pn;
-    const int room_n = pos, room_p = last - pos;
-    const long long oa = kAdjacent ? -1 : da, ob = kAdjacent ? 1 : db;
-    for (int k = 1; k <= max_dist; ++k) {
-        const bool an = rn == 0, ap = rp == 0;
-        if (k <= room_n)
-            pn -= stride;
-        if (k <= room_p)
-            pp += stride;
-        const float zcn = an ? __ldg(pn) : 0.0f;
-        const float zan = an && use_a ? __ldg(pn + oa) : 0.0f;
-        const float zbn = an && use_b ? __ldg(pn + ob) : 0.0f;
-        const float zcp = ap ? __ldg(pp) : 0.0f;
-        const float zap = ap && use_a ? __ldg(pp + oa) : 0.0f;
-        const float zbp = ap && use_b ? __ldg(pp + ob) : 0.0f;
-        if (an) {
-            if (shadow_test(pz, zcn) != s0)
-                rn = k;
-            else if (!((use_a && shadow_test(pz, zan) != s0) || (use_b && shadow_test(pz, zbn) != s0)))
-                rn = -k;
-        }
-        if (ap) {
-            if (shadow_test(pz, zcp) != s0)
-                rp = k;
-            else if (!((use_a && shadow_test(pz, zap) != s0) || (use_b && shadow_test(pz, zbp) != s0)))
-                rp = -k;
-        }
-        if (rn != 0 && rp != 0)
-            return;
-    }
-    if (rn == 0)
-        rn = -(max_dist + 1);
-    if (rp == 0)
-        rp = -(max_dist + 1);
+    // directions as the bits of d4: 0 left, 1 right, 2 +y, 3 -y
+    const bool vert = d >= 2u, up = d == 1u || d == 2u;
+    const long long along = vert ? m.pitch : 1, across = vert ? 1 : m.pitch;
+    EdgeWalk w;
+    w.p = p;
+    w.step = up ? along : -along;
+    // sides: the rows j + 1, j - 1 of a walk along x, the columns i + 1, i - 1 of one along y
+    w.side = (d4 & (vert ? 2u : 4u)) ? across : -across;
+    const int room = vert ? (up ? m.height - 1 - j : j) : (up ? m.width - 1 - i : i);
+    w.last = min(room, max_dist);
+    return w;
 }
 
-// The walks along x from texel (i, j): rows j, j+1 (shared +y) and j-1
-// (shared -y).
-__device__ __forceinline__ void walks_x(const MapDev &m, int i, int j, float pz, int s0,
-                                        bool up, bool down, int max_dist, int &rn, int &rp)
+// Walk results of the fragment at texel (i, j): rxn, rxp along x towards
+// lower and higher columns, ryn, ryp along y towards lower and higher rows.
+__device__ __forceinline__ void edge_walks(const MapDev &m, int i, int j, float pz, bool lit, unsigned d4,
+                                           int max_dist, int &rxn, int &rxp, int &ryn, int &ryp)
 {
-    const float *row = m.depth + (long long)j * m.pitch;
-    const long long du = j < m.height - 1 ? m.pitch : 0, dd = j > 0 ? -m.pitch : 0;
-    walk_pair<false>(row, du, dd, 1, i, m.width - 1, up, down, pz, s0, max_dist, rn, rp);
-}
-
-// The walks along y from texel (i, j): columns i, i-1 (shared left) and i+1
-// (shared right).
-__device__ __forceinline__ void walks_y(const MapDev &m, int i, int j, float pz, int s0,
-                                        bool left, bool right, int max_dist, int &rn, int &rp)
-{
-    walk_pair<true>(m.depth + i, 0, 0, m.pitch, j, m.height - 1, left, right, pz, s0, max_dist, rn, rp);
-}
-
-// Walks through the map's texture view, S steps per iteration (S even).
-// A 2x2 gather returns two consecutive texels of the walk's line and of one
-// neighbouring line, so an iteration takes S steps of a direction with S/2
-// gathers per side line in use (one side: S/2, both: S).  The texture
-// clamps to the edge as the scalar walk clamps its indices, so every step
-// reads the texels walk_pair reads; steps past an end or past max_dist are
-// fetched but not tested.  Gather order: x = (lo col, hi row), y = (hi, hi),
-// z = (hi, lo), w = (lo, lo); a gather at (X, Y) covers columns X-1, X and
-// rows Y-1, Y.  Used by RPCF for k != 3, whose drains it speeds up (against
-// the scalar walk stepping one pointer per direction: k = 1 / 7 at 128.4 /
-// 11.1 against 124.1 / 10.9 Gfrag/s, k = 3 at 40.25 against 40.6); the
-// batched kernel keeps the scalar walk (C5 0.351 vs 0.385 ms on 8 frames,
-// C4 94 vs 107 us per frame, measured against the earlier scalar walk).
-
-template <int S>
-__device__ __forceinline__ void walk_steps(const float (&zl)[S], const float (&za)[S], const float (&zb)[S],
-                                           bool use_a, bool use_b, float pz, int s0, int k, int max_dist, int &r)
-{
-#pragma unroll
-    for (int t = 0; t < S; ++t) {
-        if (r == 0 && k + t <= max_dist) {
-            if (shadow_test(pz, zl[t]) != s0)
-                r = k + t;
-            else if (!((use_a && shadow_test(pz, za[t]) != s0) || (use_b && shadow_test(pz, zb[t]) != s0)))
-                r = -(k + t);
-        }
-    }
-}
-
-// Along x from texel (i, j): line row j, sides rows j+1 (up) and j-1 (down).
-template <int S>
-__device__ __forceinline__ void walks_x_tex(const MapDev &m, int i, int j, float pz, int s0, bool up, bool down,
-                                            int max_dist, int &rn, int &rp)
-{
-    rn = 0;
-    rp = 0;
-    const float fj = (float)j;
-    const bool hi_pair = up || !down;      // the line from the rows j, j+1 gather unless only j-1 is in use
-    for (int k = 1; k <= max_dist; k += S) {
-        const bool on = rn == 0, op = rp == 0;
-        float ln[S], la[S], lb[S], lp[S], pa[S], pb[S];
-#pragma unroll
-        for (int g = 0; g < S / 2; ++g) {
-            // +x: columns i+k+2g (lo, step k+2g) and i+k+2g+1 (hi)
-            const float xp = (float)(i + k + 2 * g + 1);
-            float4 pu = make_float4(0.0f, 0.0f, 0.0f, 0.0f), pd = pu;
-            if (op && hi_pair)
-                pu = tex2Dgather<float4>(m.tex, xp, fj + 1.0f, 0);
-            if (op && down)
-                pd = tex2Dgather<float4>(m.tex, xp, fj, 0);
-            lp[2 * g] = hi_pair ? pu.w : pd.x;
-            lp[2 * g + 1] = hi_pair ? pu.z : pd.y;
-            pa[2 * g] = pu.x;
-            pa[2 * g + 1] = pu.y;
-            pb[2 * g] = pd.w;
-            pb[2 * g + 1] = pd.z;
-            // -x: columns i-k-2g (hi, step k+2g) and i-k-2g-1 (lo)
-            const float xn = (float)(i - k - 2 * g);
-            float4 nu = make_float4(0.0f, 0.0f, 0.0f, 0.0f), nd = nu;
-            if (on && hi_pair)
-                nu = tex2Dgather<float4>(m.tex, xn, fj + 1.0f, 0);
-            if (on && down)
-                nd = tex2Dgather<float4>(m.tex, xn, fj, 0);
-            ln[2 * g] = hi_pair ? nu.z : nd.y;
-            ln[2 * g + 1] = hi_pair ? nu.w : nd.x;
-            la[2 * g] = nu.y;
-            la[2 * g + 1] = nu.x;
-            lb[2 * g] = nd.z;
-            lb[2 * g + 1] = nd.w;
-        }
-        walk_steps<S>(ln, la, lb, up, down, pz, s0, k, max_dist, rn);
-        walk_steps<S>(lp, pa, pb, up, down, pz, s0, k, max_dist, rp);
-        if (rn != 0 && rp != 0)
+    const unsigned open = (((d4 & 12u) ? 3u : 0u) | ((d4 & 3u) ? 12u : 0u)) & ~d4;
+    const unsigned lo = open & (0u - open), hi = open & ~lo;       // walk A's direction, walk B's (or none)
+    const bool two = (d4 & 3u) == 3u || (d4 & 12u) == 12u;         // both side lines in use
+    const float *p = m.depth + (long long)j * m.pitch + i;
+    EdgeWalk A = edge_walk(m, p, i, j, __ffs(lo) - 1, d4, max_dist);
+    EdgeWalk B = edge_walk(m, p, i, j, __ffs(hi) - 1, d4, max_dist);
+    if (lo == 0u)
+        A.last = 0;
+    if (hi == 0u)
+        B.last = 0;
+    int ra = -(max_dist + 1), rb = ra;
+    for (int k = 1;; ++k) {
+        const bool a = k <= A.last, b = k <= B.last;
+        if (!a && !b)
             break;
-    }
-    rn = rn == 0 ? -(max_dist + 1) : rn;
-    rp = rp == 0 ? -(max_dist + 1) : rp;
-}
-
-// Along y from texel (i, j): line column i, sides columns i-1 (left) and
-// i+1 (right).
-template <int S>
-__device__ __forceinline__ void walks_y_tex(const MapDev &m, int i, int j, float pz, int s0, bool left, bool right,
-                                            int max_dist, int &rn, int &rp)
-{
-    rn = 0;
-    rp = 0;
-    const float fi = (float)i;
-    const bool lo_pair = left || !right;   // the line from the columns i-1, i gather unless only i+1 is in use
-    for (int k = 1; k <= max_dist; k += S) {
-        const bool on = rn == 0, op = rp == 0;
-        float ln[S], la[S], lb[S], lp[S], pa[S], pb[S];
-#pragma unroll
-        for (int g = 0; g < S / 2; ++g) {
-            // +y: rows j+k+2g (lo, step k+2g) and j+k+2g+1 (hi)
-            const float yp = (float)(j + k + 2 * g + 1);
-            float4 pl = make_float4(0.0f, 0.0f, 0.0f, 0.0f), pr = pl;
-            if (op && lo_pair)
-                pl = tex2Dgather<float4>(m.tex, fi, yp, 0);
-            if (op && right)
-                pr = tex2Dgather<float4>(m.tex, fi + 1.0f, yp, 0);
-            lp[2 * g] = lo_pair ? pl.z : pr.w;
-            lp[2 * g + 1] = lo_pair ? pl.y : pr.x;
-            pa[2 * g] = pl.w;
-            pa[2 * g + 1] = pl.x;
-            pb[2 * g] = pr.z;
-            pb[2 * g + 1] = pr.y;
-            // -y: rows j-k-2g (hi, step k+2g) and j-k-2g-1 (lo)
-            const float yn = (float)(j - k - 2 * g);
-            float4 nl = make_float4(0.0f, 0.0f, 0.0f, 0.0f), nr = nl;
-            if (on && lo_pair)
-                nl = tex2Dgather<float4>(m.tex, fi, yn, 0);
-            if (on && right)
-                nr = tex2Dgather<float4>(m.tex, fi + 1.0f, yn, 0);
-            ln[2 * g] = lo_pair ? nl.y : nr.x;
-            ln[2 * g + 1] = lo_pair ? nl.z : nr.w;
-            la[2 * g] = nl.x;
-            la[2 * g + 1] = nl.w;
-            lb[2 * g] = nr.y;
-            lb[2 * g + 1] = nr.z;
+        A.p += A.step;
+        B.p += B.step;
+        const float la = a ? __ldg(A.p) : 0.0f;
+        const float lb = b ? __ldg(B.p) : 0.0f;
+        const float sa = a ? __ldg(A.p + A.side) : 0.0f;
+        const float sb = b ? __ldg(B.p + B.side) : 0.0f;
+        // a texel's test differs from the fragment's: the walk's texel (the
+        // walk ends), its side texel (the walk continues the edge)
+        const bool ea = (pz > la) == lit, eb = (pz > lb) == lit;
+        bool ca = (pz > sa) == lit, cb = (pz > sb) == lit;
+        if (two) {
+            if (a && !ca)
+                ca = (pz > __ldg(A.p - A.side)) == lit;
+            if (b && !cb)
+                cb = (pz > __ldg(B.p - B.side)) == lit;
         }
-        walk_steps<S>(ln, la, lb, left, right, pz, s0, k, max_dist, rn);
-        walk_steps<S>(lp, pa, pb, left, right, pz, s0, k, max_dist, rp);
-        if (rn != 0 && rp != 0)
-            break;
+        if (a && (ea || !ca)) {
+            ra = ea ? k : -k;
+            A.last = 0;
+        }
+        if (b && (eb || !cb)) {
+            rb = eb ? k : -k;
+            B.last = 0;
+        }
     }
-    rn = rn == 0 ? -(max_dist + 1) : rn;
-    rp = rp == 0 ? -(max_dist + 1) : rp;
+    rxn = lo == 1u ? ra : (d4 & 1u) ? 1 : -1;
+    rxp = lo == 2u ? ra : hi == 2u ? rb : (d4 & 2u) ? 1 : -1;
+    ryp = lo == 4u ? ra : hi == 4u ? rb : (d4 & 4u) ? 1 : -1;
+    ryn = lo == 8u ? ra : hi == 8u ? rb : (d4 & 8u) ? 1 : -1;
 }
 
 // Eq. 5 and the normalisation along one axis: the position of the fragment
@@ -480,9 +374,8 @@ __device__ __forceinline__ bool classify(const MapDev &m, float x, float y, floa
 }
 
 // Steps 3-4 for one edge fragment at texel-space position (u, v)
-// (recomputes its texel).  TEX_STEPS > 0: walk through the map's texture
-// view (when it has one), TEX_STEPS steps per iteration.
-template <int MODE, int TEX_STEPS = 0>
+// (recomputes its texel).
+template <int MODE>
 __device__ __forceinline__ void resolve_edge_uv(const MapDev &m, float u, float v, float pz,
                                                 uint32_t bits, int max_dist, FragResult &r)
 {
@@ -490,27 +383,16 @@ __device__ __forceinline__ void resolve_edge_uv(const MapDev &m, float u, float 
     float fx, fy;
     texel_of(u, m.width, i, fx);
     texel_of(v, m.height, j, fy);
-    int s0 = bits & 1;
-    bool dl = (bits >> 1) & 1, dr = (bits >> 2) & 1, du = (bits >> 3) & 1, dd = (bits >> 4) & 1;
+    const int s0 = bits & 1;
+    const unsigned d4 = (bits >> 1) & 15u;
     // computeFragmentDistanceToSE: the four walks -x, +x, -y, +y
     int rxn, rxp, ryn, ryp;
-    bool done = false;
-    if constexpr (TEX_STEPS > 0) {
-        if (m.tex) {
-            walks_x_tex<TEX_STEPS>(m, i, j, pz, s0, du, dd, max_dist, rxn, rxp);
-            walks_y_tex<TEX_STEPS>(m, i, j, pz, s0, dl, dr, max_dist, ryn, ryp);
-            done = true;
-        }
-    }
-    if (!done) {
-        walks_x(m, i, j, pz, s0, du, dd, max_dist, rxn, rxp);
-        walks_y(m, i, j, pz, s0, dl, dr, max_dist, ryn, ryp);
-    }
+    edge_walks(m, i, j, pz, s0 != 0, d4, max_dist, rxn, rxp, ryn, ryp);
     int ex = (rxn > 0) + (rxp > 0);
     int ey = (ryn > 0) + (ryp > 0);
     float nx = axis_position(rxn, rxp, fx);
     float ny = axis_position(ryn, ryp, fy);
-    bool dx3 = dl && dr, dy3 = du && dd;
+    const bool dx3 = (d4 & 3u) == 3u, dy3 = (d4 & 12u) == 12u;
     r.code = (uint16_t)(r.code | (ex << 5) | (ey << 7) | (1 << 9));
     if (MODE & 1)
         r.sil = s0 ? silhouette(dx3, dy3, ex, ey, nx, ny) : 0.0f;

@@ -242,9 +242,7 @@ rpcf_kernel(const MapDev m, const float *__restrict__ x, const float *__restrict
                 } else {
                     classify_uv<2, false>(m, ua, vb, pz, r, bits);    // the sample's discontinuity again
                 }
-                // walks through the texture view (two steps per gather), except
-                // for k = 3, where the scalar walk measured 1 % faster
-                resolve_edge_uv<2, K == 3 ? 0 : 2>(m, ua, vb, pz, bits, max_dist, r);
+                resolve_edge_uv<2>(m, ua, vb, pz, bits, max_dist, r);
                 if (K == 1) {
                     vis[i] = r.fil;
                 } else {
@@ -342,7 +340,7 @@ rpcf_kernel(const MapDev m, const float *__restrict__ x, const float *__restrict
                     uint32_t bits = 0;
                     const float ua = __fadd_rn(u, (float)(q % K - R)), vb = __fadd_rn(v, (float)(q / K - R));
                     if (classify_uv<2, false>(m, ua, vb, ze, r, bits))
-                        resolve_edge_uv<2, K == 3 ? 0 : 2>(m, ua, vb, ze, bits, max_dist, r);
+                        resolve_edge_uv<2>(m, ua, vb, ze, bits, max_dist, r);
                     if (r.fil != r.fil)
                         nan = true;               // a NaN answer (NaN or infinite coordinates)
                     else
