@@ -276,9 +276,11 @@ typedef struct {
      * bit 10 set and no end counts (bits 5-9 clear). */
     const void *surrogate;
     float guard_tau;
-    int32_t chunk_tiles;           /* 128-fragment warp tiles a warp claims at a time from the
-                                    * work counter: 1, 2, 4 or 8; 0 = chosen from the batch size
-                                    * (8 when every warp gets about eight claims, halved below) */
+    int32_t chunk_tiles;           /* 128-fragment warp tiles a warp claims at a time from a
+                                    * work counter: 1, 2, 4 or 8; 0 = chosen by the library (1 in
+                                    * a workspace of the size rbsm_batch_workspace_size gives; in
+                                    * a smaller one, which holds a single counter, 4 when every
+                                    * warp gets about eight claims, halved below) */
     int32_t flags;                 /* 0 or RBSM_BATCH_PLAIN_LOADS */
 } rbsm_batch;
 
@@ -287,17 +289,18 @@ typedef struct {
 #define RBSM_BATCH_PLAIN_LOADS 1
 
 /*
- * Device workspace a batch needs (a work counter and a status word), in
+ * Device workspace a batch needs (work counters and a status word), in
  * bytes; the caller allocates it (256-byte aligned) and may reuse it for any
- * later batch that is not in flight at the same time.
+ * later batch that is not in flight at the same time.  A workspace of 256
+ * bytes or more is accepted too: the warps then share one work counter.
  */
 int rbsm_batch_workspace_size(const rbsm_batch *batch, size_t *bytes);
 
 /*
  * Enqueue one batched launch: a memset of the workspace followed by one
  * persistent kernel whose warps take chunks of 1 to 8 tiles of 128
- * fragments (in job order; the chunk is as large as leaves every warp
- * about eight claims) from an atomic counter in the workspace.
+ * fragments (in job order, see chunk_tiles) from atomic counters in the
+ * workspace.
  * The descriptors are copied into the launch parameters, so the host arrays
  * may be reused as soon as the call returns.  Errors: RBSM_ERR_ARG as for
  * rbsm_visibility applied to every map and job, or a map index out of range;
@@ -313,7 +316,7 @@ int rbsm_batch_run(const rbsm_batch *batch, void *workspace, size_t workspace_by
  * that must not allocate while frames are in flight.  The paper has no
  * counterpart; this is a convenience of the library.
  *
- * The scratch rbsm_batch_run keeps in the caller's workspace (work counter,
+ * The scratch rbsm_batch_run keeps in the caller's workspace (work counters,
  * status word, surrogate counters) lives instead in one device array
  * compiled into the library, RBSM_NOALLOC_SCRATCH_BYTES bytes, which every
  * GPU that loads the library holds until the process exits.  The call
@@ -330,7 +333,7 @@ int rbsm_batch_run(const rbsm_batch *batch, void *workspace, size_t workspace_by
  * (rbsm_batch_workspace_size) exceeds the array is rejected with
  * RBSM_ERR_WORKSPACE; other errors as for rbsm_batch_run.
  */
-#define RBSM_NOALLOC_SCRATCH_BYTES 256
+#define RBSM_NOALLOC_SCRATCH_BYTES 4096
 int rbsm_batch_run_noalloc(const rbsm_batch *batch, void *stream);
 
 /* The surrogate counters (as rbsm_batch_surrogate_counts) of the last
@@ -360,7 +363,7 @@ int rbsm_batch_graph_destroy(rbsm_graph graph);
  *   - 7 (CTA size, CTAs per SM) pairs: 128 threads at its occupancy limit;
  *     256 threads at 2, 3, 4 and 5 (occupancy limit) CTAs per SM; 512
  *     threads at 1 and 2;
- *   - 4 claim sizes: 1, 2, 4 and 8 warp tiles per claim of the work counter;
+ *   - 4 claim sizes: 1, 2, 4 and 8 warp tiles per claim of a work counter;
  *   - when any map carries a texture: texture gathers or plain loads for the
  *     four-neighbourhood;
  * with `repeats` launches each after one warm-up, on `stream`, and returns

@@ -1,6 +1,6 @@
 // Batched evaluation: many shadow maps x many fragment sets in one
-// persistent launch (host side; the kernel is in rbsm_batch_kernel.cuh).  CTAs take (job, tile) work items from an atomic
-// counter in the caller's workspace, so maps of very different sizes and
+// persistent launch (host side; the kernel is in rbsm_batch_kernel.cuh).  CTAs take (job, tile) work items from atomic
+// counters in the caller's workspace, so maps of very different sizes and
 // views of very different resolutions share the GPU without a launch per
 // pair and without idle SMs at the end of small jobs.
 #include <cuda_runtime.h>
@@ -88,12 +88,12 @@ int shape_for(const BatchArgs &args, int ctas_per_sm, int chunk_req, int umode, 
     const int sms = device_sm_count();
     if (sms <= 0)
         return cuda_fail(cudaErrorNoDevice);
-    // about 8 claims per warp: chunks of 8 tiles when there is work enough,
-    // smaller ones (a power of two, down to 1) for launches of a few tiles
-    // per warp, where the last chunks would otherwise leave warps idle
+    // claims of one tile from several counters; of up to 4 tiles from a
+    // single one (about 8 claims per warp, fewer tiles each in launches of a
+    // few tiles per warp, where the last chunks would leave warps idle)
     long long grid = (long long)sms * occ;
     const long long warps = grid * (kThreads / 32);
-    int chunk = kMaxChunkTiles;
+    int chunk = args.n_counters > 1 ? 1 : 4;
     while (chunk > 1 && args.total_tiles < 8LL * chunk * warps)
         chunk >>= 1;
     if (chunk_req > 0)
@@ -104,7 +104,9 @@ int shape_for(const BatchArgs &args, int ctas_per_sm, int chunk_req, int umode, 
         grid = blocks_needed;
     if (grid < 1)
         grid = 1;
-    *out = LaunchShape{fn, kThreads, (unsigned)grid, smem, chunk};
+    // every counter in use has a CTA of its own
+    const int counters = grid >= kCounters ? args.n_counters : 1;
+    *out = LaunchShape{fn, kThreads, (unsigned)grid, smem, chunk, counters};
     return RBSM_OK;
 }
 
@@ -150,7 +152,10 @@ int launch_shape(const BatchArgs &args, int threads, int ctas_per_sm, int chunk,
 int launch_kernel(BatchArgs &args, const LaunchShape &sh, cudaStream_t stream)
 {
     args.chunk_tiles = sh.chunk;
+    const int have = args.n_counters;
+    args.n_counters = sh.counters;
     sh.kernel<<<sh.grid, sh.threads, sh.smem, stream>>>(args);
+    args.n_counters = have;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return cuda_fail(e);
@@ -233,15 +238,18 @@ int prepare_batch(const rbsm_batch *b, BatchArgs &a, int *threads)
 
 int check_workspace(const void *ws, size_t bytes)
 {
-    if (!ws || bytes < kWorkspaceBytes || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0)
+    if (!ws || bytes < kMinWorkspaceBytes || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0)
         return RBSM_ERR_WORKSPACE;
     return RBSM_OK;
 }
 
 // Workspace layout: [0] work counter (u64), [8] status word (int),
-// [16] surrogate answers (u64), [24] surrogate fallbacks (u64).
-void bind_workspace(BatchArgs &a, void *ws)
+// [16] surrogate answers (u64), [24] surrogate fallbacks (u64); in a
+// workspace of kWorkspaceBytes the other counters at every kCounterStride
+// bytes, in a smaller one the first counter alone.
+void bind_workspace(BatchArgs &a, void *ws, size_t bytes)
 {
+    a.n_counters = bytes >= kWorkspaceBytes ? kCounters : 1;
     a.counter = reinterpret_cast<unsigned long long *>(ws);
     a.status = reinterpret_cast<int *>(reinterpret_cast<char *>(ws) + 8);
     a.stats = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(ws) + 16);
@@ -252,7 +260,8 @@ int enqueue_batch(BatchArgs &a, const LaunchShape &sh, void *ws, cudaStream_t s)
 {
     if (a.total_tiles == 0)
         return RBSM_OK;
-    cudaError_t e = cudaMemsetAsync(ws, 0, 32, s);
+    const size_t used = (size_t)(sh.counters - 1) * kCounterStride + 32;
+    cudaError_t e = cudaMemsetAsync(ws, 0, used, s);
     if (e != cudaSuccess)
         return cuda_fail(e);
     return launch_kernel(a, sh, s);
@@ -287,7 +296,7 @@ int rbsm_batch_run(const rbsm_batch *batch, void *workspace, size_t workspace_by
         return rc;
     if ((rc = rbsm::check_workspace(workspace, workspace_bytes)) != RBSM_OK)
         return rc;
-    rbsm::bind_workspace(args, workspace);
+    rbsm::bind_workspace(args, workspace, workspace_bytes);
     if (args.total_tiles == 0)
         return RBSM_OK;
     rbsm::LaunchShape sh;
@@ -309,8 +318,8 @@ int rbsm_batch_graph_create(const rbsm_batch *batch, void *workspace, size_t wor
         return rc;
     if ((rc = rbsm::check_workspace(workspace, workspace_bytes)) != RBSM_OK)
         return rc;
-    rbsm::bind_workspace(args, workspace);
-    rbsm::LaunchShape sh{nullptr, 256, 1, 0, 1};
+    rbsm::bind_workspace(args, workspace, workspace_bytes);
+    rbsm::LaunchShape sh{nullptr, 256, 1, 0, 1, 1};
     if (args.total_tiles > 0 &&
         (rc = rbsm::launch_shape(args, threads, batch->ctas_per_sm, batch->chunk_tiles, &sh)) != RBSM_OK)
         return rc;
@@ -380,7 +389,7 @@ int rbsm_batch_autotune(const rbsm_batch *batch, void *workspace, size_t workspa
         return rc;
     if ((rc = rbsm::check_workspace(workspace, workspace_bytes)) != RBSM_OK)
         return rc;
-    rbsm::bind_workspace(args, workspace);
+    rbsm::bind_workspace(args, workspace, workspace_bytes);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     best->tile_threads = 256;
     best->ctas_per_sm = 0;
@@ -534,14 +543,14 @@ extern "C" int rbsm_batch_run_noalloc(const rbsm_batch *batch, void *stream)
     void *scratch = nullptr;
     if ((rc = noalloc_scratch_for_current_device(&scratch)) != RBSM_OK)
         return rc;
-    rbsm::bind_workspace(args, scratch);
+    rbsm::bind_workspace(args, scratch, RBSM_NOALLOC_SCRATCH_BYTES);
     if (args.total_tiles == 0)
         return RBSM_OK;
     rbsm::LaunchShape sh;
     if ((rc = rbsm::launch_shape(args, threads, batch->ctas_per_sm, batch->chunk_tiles, &sh)) != RBSM_OK)
         return rc;
     // enqueue_batch clears the counters that must start at zero (a memset of
-    // the array's first 32 bytes, stream-ordered before the kernel)
+    // the array, stream-ordered before the kernel)
     return rbsm::enqueue_batch(args, sh, scratch, reinterpret_cast<cudaStream_t>(stream));
 }
 

@@ -20,6 +20,7 @@ struct LaunchShape {
     unsigned grid;
     size_t smem;
     int chunk;                      // warp tiles per claim (BatchArgs::chunk_tiles)
+    int counters;                   // work counters in use (BatchArgs::n_counters)
 };
 
 // Validate a batch and fill the kernel arguments (everything but the
@@ -29,9 +30,10 @@ int prepare_batch(const rbsm_batch *b, BatchArgs &a, int *threads);
 // tiles per claim (1, 2, 4, 8), 0 = chosen from the batch size.
 int launch_shape(const BatchArgs &args, int threads, int ctas_per_sm, int chunk, LaunchShape *out);
 int check_workspace(const void *ws, size_t bytes);
-// Point the kernel arguments at the counter, status word and statistics of
-// a workspace.
-void bind_workspace(BatchArgs &a, void *ws);
+// Point the kernel arguments at the counters, status word and statistics of
+// a workspace of `bytes` bytes (before launch_shape, whose claim size depends
+// on the number of counters).
+void bind_workspace(BatchArgs &a, void *ws, size_t bytes);
 // Enqueue the workspace memset and the kernel (nothing for an empty batch);
 // sets a.chunk_tiles from the shape.
 int enqueue_batch(BatchArgs &a, const LaunchShape &sh, void *ws, cudaStream_t s);

@@ -313,7 +313,7 @@ int run_map(rbsm_stager_s *st, const rbsm_batch *b, int map_index, const int *id
     int threads = 0;
     if ((rc = prepare_batch(&db, args, &threads)) != RBSM_OK)
         return rc;
-    bind_workspace(args, s.ws);
+    bind_workspace(args, s.ws, kWorkspaceBytes);
     LaunchShape sh;
     if ((rc = launch_shape(args, threads, db.ctas_per_sm, db.chunk_tiles, &sh)) != RBSM_OK)
         return rc;
