@@ -319,6 +319,22 @@ __device__ __forceinline__ bool classify_from(float pz, float zc, float zl, floa
     return edge;
 }
 
+// The texel of position (u, v) and its four neighbours through the map's
+// texture.  Texel coordinates in float (clamp(floor(u)) is an integer-valued
+// float, exact below 2^24), then two 2x2 gathers (point sampling, clamp to
+// edge, unnormalised coordinates; the footprint of a gather at (u, v) is
+// columns u-1, u and rows v-1, v): a at (i, j) columns i-1..i, rows j-1..j; b
+// at (i+1, j+1) columns i..i+1, rows j..j+1.  Gather order: x = (lo col, hi
+// row), y = (hi, hi), z = (hi, lo), w = (lo, lo), so the texel is a.y, its
+// left, right, +y and -y neighbours a.x, b.z, b.x, a.z.
+__device__ __forceinline__ void gather_cross(const MapDev &m, float u, float v, float4 &a, float4 &b)
+{
+    const float ci = fminf(fmaxf(floorf(u), 0.0f), (float)(m.width - 1));
+    const float cj = fminf(fmaxf(floorf(v), 0.0f), (float)(m.height - 1));
+    a = tex2Dgather<float4>(m.tex, ci, cj, 0);
+    b = tex2Dgather<float4>(m.tex, ci + 1.0f, cj + 1.0f, 0);
+}
+
 // Steps 1-2 for one fragment: texel, shadow test, four-neighbourhood.
 // Returns true when the fragment needs the edge walk for this mode; packs
 // s0 and the four directions into `bits` (bit 0 = s0, bits 1-4 = left,
@@ -331,17 +347,8 @@ __device__ __forceinline__ bool classify_uv(const MapDev &m, float u, float v, f
                                             FragResult &r, uint32_t &bits)
 {
     if (m.tex) {
-        // Texel coordinates in float (clamp(floor(u)) is an integer-valued
-        // float, exact below 2^24), then two 2x2 gathers (point sampling,
-        // clamp to edge, unnormalised coordinates; the footprint of a gather
-        // at (u, v) is columns u-1, u and rows v-1, v): at (i, j) columns
-        // i-1..i, rows j-1..j; at (i+1, j+1) columns i..i+1, rows j..j+1.
-        // Gather order: x = (lo col, hi row), y = (hi, hi), z = (hi, lo),
-        // w = (lo, lo).
-        const float ci = fminf(fmaxf(floorf(u), 0.0f), (float)(m.width - 1));
-        const float cj = fminf(fmaxf(floorf(v), 0.0f), (float)(m.height - 1));
-        const float4 a = tex2Dgather<float4>(m.tex, ci, cj, 0);
-        const float4 b = tex2Dgather<float4>(m.tex, ci + 1.0f, cj + 1.0f, 0);
+        float4 a, b;
+        gather_cross(m, u, v, a, b);
         return classify_from<MODE, CODES>(pz, a.y, a.x, b.z, b.x, a.z, r, bits);
     }
     int i, j;
@@ -605,7 +612,31 @@ __device__ __forceinline__ void classify_warp_tile(const MapDev &m, const WarpTi
     bool edge[kPerThread];
     // classify the lane's four fragments first (no warp-wide step in between,
     // so all their texel loads are issued back to back) ...
-    if (t.vec) {
+    if (m.tex) {
+        // one branch for the four fragments' eight gathers: tested per
+        // fragment, the texture handle put a branch between one fragment's
+        // gathers and the next one's (depth buffers, 4 frames of 3840x2160
+        // pixels: 241 against 219 us; planes, 8 frames in one launch: 369
+        // against 349 us).  Bound: a gather's four components take the
+        // texture path about 16 cycles to write back for a warp, 26 us of a
+        // 3840x2160 frame; fetching the right and upper neighbours one by one
+        // instead (two point fetches, or two loads, for the second gather)
+        // was slower: 458 and 494 us for the 8 frames.
+        // A partial tile's lanes past its end hold zeros and are masked after.
+        const float W = (float)m.width, H = (float)m.height;
+        float4 a[kPerThread], b[kPerThread];
+#pragma unroll
+        for (int e = 0; e < kPerThread; ++e)
+            gather_cross(m, __fmul_rn(c.x[e], W), __fmul_rn(c.y[e], H), a[e], b[e]);
+#pragma unroll
+        for (int e = 0; e < kPerThread; ++e)
+            edge[e] = classify_from<MODE, CODES>(c.z[e], a[e].y, a[e].x, b[e].z, b[e].x, a[e].z, r[e], bits[e]);
+        if (!t.vec) {
+#pragma unroll
+            for (int e = 0; e < kPerThread; ++e)
+                edge[e] = edge[e] && (int)lane + 32 * e < t.count;
+        }
+    } else if (t.vec) {
 #pragma unroll
         for (int e = 0; e < kPerThread; ++e)
             edge[e] = classify<MODE, CODES>(m, c.x[e], c.y[e], c.z[e], r[e], bits[e]);
