@@ -4,12 +4,12 @@
 // samples at its texel-space position shifted by whole texels, (u + a,
 // v + b), each with the fragment's depth.
 //
-// Same warp-tile scheme as the other kernels, with the sample as the unit
-// of deferred work: a lane classifies its fragments' samples (two texture
-// gathers or five loads each); off-edge samples add their shadow test at
-// once, edge samples go to the warp's queue (fragment and sample index; for
-// k = 3 with the fragment's shadow tests, else the drain classifies the
-// sample again) and are walked 32 at a time on full warps.  For k > 1 a
+// The sample is the unit of deferred work: a lane classifies its fragment's
+// samples (two texture gathers or five loads each, or all from one block,
+// below); off-edge samples add their shadow test at once, edge samples go to
+// the warp's queue (fragment and sample index; for k = 3 with the fragment's
+// shadow tests, else the drain classifies the sample again) and are walked
+// 32 at a time on full warps.  For k > 1 a
 // fragment with edge samples keeps its sum in the output plane as a
 // fixed-point integer (each sample answer rounded to 2^-F, F = 24 / 22 / 20
 // for k = 3 / 5 / 7) below a count of its samples still to come; the adds
@@ -19,8 +19,7 @@
 // (below) walks its own samples, so no second pass is needed.  For k = 1
 // there is nothing to add and the answers are stored as floats
 // (rsmss_filter's bits).  Because the answers do not depend on the order of
-// the work, rbsm_rpcf_ws can hand the tiles out from a counter (balance
-// between warps) and give the same bits as rbsm_rpcf's fixed partition.
+// the work, the warps of a CTA share its strips as they come free.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -32,7 +31,12 @@
 namespace rbsm {
 namespace {
 
-constexpr int kRpcfThreads = 256;
+// One CTA of 32 warps per SM for k > 1 (two of 16 warps: 143.8 against 134.5
+// us at k = 3, four of 8: 159.7; the larger the CTA, the more strips its
+// warps share out), and for k = 1, whose kernel fits 48 registers, two of 20
+// (61.1 us with one of 32, 56.7 with these).  3840x2160 fragments.
+template <int K>
+constexpr int kRpcfThreads = K == 1 ? 640 : 1024;
 
 // The fixed-point layout of a pending fragment: F fraction bits per sample
 // answer, the sum (at most K^2 * 2^F) below bit kCount, and the number of
@@ -156,7 +160,19 @@ __device__ __forceinline__ void block_bits(const MapDev &m, float u, float v, fl
 #pragma unroll
     for (int y = 0; y < B; ++y)
         rows[y] = 0u;
-    if constexpr (K == 3) {
+    if (!m.tex) {
+        // plain loads, a row of the block at a time (1279x717 fragments, k =
+        // 3: 61.7 us against 99 us when each lane classified and walked its
+        // fragment's samples one after the other)
+        const float *row = m.depth + (long long)((int)floorf(v) - R - 1) * m.pitch + ((int)floorf(u) - R - 1);
+#pragma unroll
+        for (int y = 0; y < B; ++y) {
+#pragma unroll
+            for (int x = 0; x < B; ++x)
+                rows[y] |= (uint32_t)!(pz > __ldg(row + x)) << x;
+            row += m.pitch;
+        }
+    } else if constexpr (K == 3) {
         gather_bits<K>(m, gx, gy, 0, 0, pz, rows);
         gather_bits<K>(m, gx, gy, 2, 0, pz, rows);
         gather_bits<K>(m, gx, gy, 3, 1, pz, rows);
@@ -174,47 +190,50 @@ __device__ __forceinline__ void block_bits(const MapDev &m, float u, float v, fl
     }
 }
 
+// Persistent warps work on strips of 32 consecutive fragments, one per lane.
+// A CTA owns every gridDim.x-th run of kRun strips (its warps' loads stay
+// near each other), and its warps take them one at a time from a counter in
+// shared memory, so that a strip along a shadow edge, whose samples all walk,
+// holds up one warp while the others take the strips after it.
+//
+// Bound: the texture path's write-back of the block's gathers (7 for k = 3,
+// about 16 cycles each for a warp: 92 us of a 3840x2160 frame), then the
+// rounds of the longest walks.  A warp used to own a tile of 128 fragments
+// (up to 1152 samples, 36 rounds, at k = 3), and the tiles came from a fixed
+// partition or one at a time from a global counter; 3840x2160 fragments on
+// an 8192^2 map, k = 1 / 3 / 5: 66 / 179 / 488 us with tiles from the
+// counter, 56.7 / 134.5 / 291 us now.
+constexpr unsigned kRun = 8;       // 16: 161.7 against 159.7 us, and 48 against 32.4 us for 320x240 fragments
+
 template <int K, int kThreads>
-__global__ void __launch_bounds__(kThreads, 1024 / kThreads)
+__global__ void __launch_bounds__(kThreads, K == 1 ? 2 : 1)
 rpcf_kernel(const MapDev m, const float *__restrict__ x, const float *__restrict__ y,
-            const float *__restrict__ z, long long n, float *__restrict__ vis, int max_dist, bool vec_planes,
-            unsigned long long *next_tile)
+            const float *__restrict__ z, long long n, float *__restrict__ vis, int max_dist)
 {
     constexpr int kWarps = kThreads / 32;
     constexpr int R = (K - 1) / 2;
     __shared__ RpcfQueue<K> wq[kWarps];
-    __shared__ float4 next[kWarps][3][32];     // the next tile's coordinates (cp.async)
+    __shared__ unsigned next;                  // strips of this CTA taken
+    if (threadIdx.x == 0)
+        next = kWarps;
+    __syncthreads();
     const unsigned lane = lane_id();
     const unsigned below = (1u << lane) - 1u;
-    const int warp = threadIdx.x >> 5;
-    const long long stride = (long long)gridDim.x * kWarps;
-    const long long tiles = (n + kWarpTile - 1) / kWarpTile;
-    long long tile = (long long)blockIdx.x * kWarps + warp;
-    if (tile >= tiles)
+    // the warp's index through a shuffle: the compiler then knows that the
+    // strip and what follows from it are the same on all lanes
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const long long strips = (n + 31) / 32;
+    // strip number k of this CTA
+    auto strip_of = [&](unsigned k) {
+        return (long long)(k / kRun) * ((long long)gridDim.x * kRun) + (long long)blockIdx.x * kRun + k % kRun;
+    };
+    long long strip = strip_of((unsigned)warp);
+    if (strip >= strips)
         return;
-    // schedule: every warp takes one tile of the first wave; after that
-    // either the static stride or, with a counter (next_tile, k > 1), one
-    // tile per claim, taken one tile ahead, so that warps whose tiles carry
-    // many edge samples do not hold up the end of the launch
-    const bool claims = K > 1 && next_tile != nullptr;
-    unsigned long long claim = 0;
-    if (claims && lane == 0)
-        claim = atomicAdd(next_tile, 1ull);
     const float W = (float)m.width, H = (float)m.height;
     // the largest floor(u), floor(v) whose block lies inside the map
     const float uhi = (float)(m.width - R - 2), vhi = (float)(m.height - R - 2);
-    const bool tex = K > 1 && m.tex != 0;
     uint32_t *acc = reinterpret_cast<uint32_t *>(vis);
-    auto io_of = [&](long long tl) {
-        WarpTileIO t;
-        t.x = x; t.y = y; t.z = z; t.sil = nullptr; t.fil = vis; t.codes = nullptr;
-        t.first = tl * kWarpTile;
-        const long long left = n - t.first;
-        t.count = left < kWarpTile ? (int)left : kWarpTile;
-        t.job = 0;
-        t.vec = vec_planes && t.count == kWarpTile;
-        return t;
-    };
     // drain rounds of 32 queued edge samples: walk, answer, add
     auto drain = [&](int &queued, bool all) {
         while (queued >= 32 || (all && queued > 0)) {
@@ -259,182 +278,168 @@ rpcf_kernel(const MapDev m, const float *__restrict__ x, const float *__restrict
             queued = base;
         }
     };
-    WarpTileIO t = io_of(tile);
-    float4 (&buf)[3][32] = next[warp];
-    stage_tile(t, lane, buf);
     int queued = 0;
+    float xn = 0.0f, yn = 0.0f, zn = 0.0f;         // this lane's fragment of the next strip
+    auto load = [&](long long st) {
+        const long long f = st * 32 + lane;
+        if (f < n) {
+            xn = __ldcs(x + f);
+            yn = __ldcs(y + f);
+            zn = __ldcs(z + f);
+        }
+    };
+    load(strip);
     for (;;) {
-        long long nt = tile + stride;
-        if (claims) {
-            nt = stride + (long long)__shfl_sync(0xffffffffu, claim, 0);
-            if (nt < tiles && lane == 0)
-                claim = atomicAdd(next_tile, 1ull);
-        }
-        const bool more = nt < tiles;
-        WarpTileIO tn;
-        LaneCoords c;
-        fetch_tile_strided(t, lane, buf, c);
-        if (more) {
-            tn = io_of(nt);
-            stage_tile(tn, lane, buf);     // next tile's copies fly during this tile
-        }
-#pragma unroll 1
-        for (int e = 0; e < kPerThread; ++e) {
-            const int s = (int)lane + 32 * e;
-            const bool valid = s < t.count;
-            const float xe = e == 0 ? c.x[0] : e == 1 ? c.x[1] : e == 2 ? c.x[2] : c.x[3];
-            const float ye = e == 0 ? c.y[0] : e == 1 ? c.y[1] : e == 2 ? c.y[2] : c.y[3];
-            const float ze = e == 0 ? c.z[0] : e == 1 ? c.z[1] : e == 2 ? c.z[2] : c.z[3];
-            const float u = __fmul_rn(xe, W), v = __fmul_rn(ye, H);
-            // all samples' texel reads first; off-edge samples add their
-            // shadow test to the base value, edge samples set their bit
-            uint64_t edges = 0;
-            uint32_t base = 0, block = 0;
-            float single = 0.0f;
-            const bool base_path = tex && valid && block_ok<K>(u, v, uhi, vhi);
-            if (base_path) {
-                uint32_t rows[K + 2];
-                block_bits<K>(m, u, v, ze, rows);
-                // a row of samples at once: sample (a, b)'s texel is block
-                // (a + 1, b + 1); it is an edge sample where one of Listing
-                // 2's four neighbours differs from it, else it adds its
-                // shadow test
-                if constexpr (K == 3) {
-                    // the whole 5 x 5 block in one word, row y at bits 5y..5y+4:
-                    // a sample differs from a neighbour one bit (left, right)
-                    // or five bits (below, above) away, so the four
-                    // comparisons of Listing 2 cover all nine samples at once
-                    const uint32_t P = rows[0] | (rows[1] << 5) | (rows[2] << 10) | (rows[3] << 15) | (rows[4] << 20);
-                    constexpr uint32_t kSamples = (7u << 6) | (7u << 11) | (7u << 16);   // rows 1-3, columns 1-3
-                    const uint32_t e = ((P ^ (P >> 1)) | (P ^ (P << 1)) | (P ^ (P >> 5)) | (P ^ (P << 5))) & kSamples;
-                    edges = e;
-                    block = P;
-                    base = (uint32_t)__popc(P & ~e & kSamples) << FixLayout<K>::kFrac;
-                } else {
-                    constexpr uint32_t mk = (1u << K) - 1u;
+        unsigned k = 0;
+        if (lane == 0)
+            k = atomicAdd(&next, 1u);
+        const long long ns = strip_of(__shfl_sync(0xffffffffu, k, 0));
+        const bool more = ns < strips;
+        const float xe = xn, ye = yn, ze = zn;
+        const long long frag = strip * 32 + lane;
+        const bool valid = frag < n;
+        if (more)
+            load(ns);                      // the next strip's loads fly during this one
+        const float u = __fmul_rn(xe, W), v = __fmul_rn(ye, H);
+        // all samples' texel reads first; off-edge samples add their
+        // shadow test to the base value, edge samples set their bit
+        uint64_t edges = 0;
+        uint32_t base = 0, block = 0;
+        float single = 0.0f;
+        const bool base_path = K > 1 && valid && block_ok<K>(u, v, uhi, vhi);
+        if (base_path) {
+            uint32_t rows[K + 2];
+            block_bits<K>(m, u, v, ze, rows);
+            // a row of samples at once: sample (a, b)'s texel is block
+            // (a + 1, b + 1); it is an edge sample where one of Listing
+            // 2's four neighbours differs from it, else it adds its
+            // shadow test
+            if constexpr (K == 3) {
+                // the whole 5 x 5 block in one word, row y at bits 5y..5y+4:
+                // a sample differs from a neighbour one bit (left, right)
+                // or five bits (below, above) away, so the four
+                // comparisons of Listing 2 cover all nine samples at once
+                const uint32_t P = rows[0] | (rows[1] << 5) | (rows[2] << 10) | (rows[3] << 15) | (rows[4] << 20);
+                constexpr uint32_t kSamples = (7u << 6) | (7u << 11) | (7u << 16);   // rows 1-3, columns 1-3
+                const uint32_t e = ((P ^ (P >> 1)) | (P ^ (P << 1)) | (P ^ (P >> 5)) | (P ^ (P << 5))) & kSamples;
+                edges = e;
+                block = P;
+                base = (uint32_t)__popc(P & ~e & kSamples) << FixLayout<K>::kFrac;
+            } else {
+                constexpr uint32_t mk = (1u << K) - 1u;
 #pragma unroll
-                    for (int b = 0; b < K; ++b) {
-                        const uint32_t c = (rows[b + 1] >> 1) & mk;
-                        const uint32_t e = (c ^ (rows[b + 1] & mk)) | (c ^ ((rows[b + 1] >> 2) & mk)) |
-                                           (c ^ ((rows[b + 2] >> 1) & mk)) | (c ^ ((rows[b] >> 1) & mk));
-                        edges |= (uint64_t)e << (K * b);
-                        base += (uint32_t)__popc(c & ~e) << FixLayout<K>::kFrac;
-                    }
+                for (int b = 0; b < K; ++b) {
+                    const uint32_t c = (rows[b + 1] >> 1) & mk;
+                    const uint32_t e = (c ^ (rows[b + 1] & mk)) | (c ^ ((rows[b + 1] >> 2) & mk)) |
+                                       (c ^ ((rows[b + 2] >> 1) & mk)) | (c ^ ((rows[b] >> 1) & mk));
+                    edges |= (uint64_t)e << (K * b);
+                    base += (uint32_t)__popc(c & ~e) << FixLayout<K>::kFrac;
                 }
-            } else if (K == 1) {
+            }
+        } else if (K == 1) {
+            FragResult r{0.0f, 0.0f, 0};
+            uint32_t bits = 0;
+            if (valid && classify_uv<2, false>(m, u, v, ze, r, bits))
+                edges = 1ull << sample_slot<K>(0);
+            single = r.fil;
+        } else if (valid) {
+            // outside the shared block (the map's border rows and
+            // columns, or a non-finite coordinate): the lane walks its
+            // own edge samples and writes the mean (rare, so the
+            // divergence costs little)
+            uint32_t sum = 0;
+            bool nan = false;
+#pragma unroll 1
+            for (int q = 0; q < K * K; ++q) {
                 FragResult r{0.0f, 0.0f, 0};
                 uint32_t bits = 0;
-                if (valid && classify_uv<2, false>(m, u, v, ze, r, bits))
-                    edges = 1ull << sample_slot<K>(0);
-                single = r.fil;
-            } else if (valid) {
-                // outside the shared block (the map's border rows and
-                // columns, or a non-finite coordinate): the lane walks its
-                // own edge samples and writes the mean (rare, so the
-                // divergence costs little)
-                uint32_t sum = 0;
-                bool nan = false;
-#pragma unroll 1
-                for (int q = 0; q < K * K; ++q) {
-                    FragResult r{0.0f, 0.0f, 0};
-                    uint32_t bits = 0;
-                    const float ua = __fadd_rn(u, (float)(q % K - R)), vb = __fadd_rn(v, (float)(q / K - R));
-                    if (classify_uv<2, false>(m, ua, vb, ze, r, bits))
-                        resolve_edge_uv<2>(m, ua, vb, ze, bits, max_dist, r);
-                    if (r.fil != r.fil)
-                        nan = true;               // a NaN answer (NaN or infinite coordinates)
-                    else
-                        sum += to_fix<K>(r.fil);
-                }
-                vis[t.first + s] = nan ? __int_as_float(0x7fc00000) : mean_of<K>(sum);
+                const float ua = __fadd_rn(u, (float)(q % K - R)), vb = __fadd_rn(v, (float)(q / K - R));
+                if (classify_uv<2, false>(m, ua, vb, ze, r, bits))
+                    resolve_edge_uv<2>(m, ua, vb, ze, bits, max_dist, r);
+                if (r.fil != r.fil)
+                    nan = true;               // a NaN answer (NaN or infinite coordinates)
+                else
+                    sum += to_fix<K>(r.fil);
             }
-            // the base value is stored before any deferred sample of this
-            // fragment can add to it ...
-            const uint32_t ne = (uint32_t)__popcll(edges);
-            if (valid) {
-                if (K == 1)
-                    vis[t.first + s] = single;
-                else if (ne != 0)
-                    acc[t.first + s] = (ne << FixLayout<K>::kCount) | base;
-                else if (base_path)
-                    vis[t.first + s] = mean_of_lit<K>(base >> FixLayout<K>::kFrac);
-            }
-            // ... then the edge samples are queued and walked whenever 32
-            // are waiting
-            if (K <= 3) {
-                // all of the lane's edge samples, placed by a prefix sum
-                uint32_t incl = ne, total = 0;
-                if (__any_sync(0xffffffffu, ne != 0)) {      // about one element in five has none
+            vis[frag] = nan ? __int_as_float(0x7fc00000) : mean_of<K>(sum);
+        }
+        // the base value is stored before any deferred sample of this
+        // fragment can add to it ...
+        const uint32_t ne = (uint32_t)__popcll(edges);
+        if (valid) {
+            if (K == 1)
+                vis[frag] = single;
+            else if (ne != 0)
+                acc[frag] = (ne << FixLayout<K>::kCount) | base;
+            else if (base_path)
+                vis[frag] = mean_of_lit<K>(base >> FixLayout<K>::kFrac);
+        }
+        // ... then the edge samples are queued and walked whenever 32
+        // are waiting
+        if (K <= 3) {
+            // all of the lane's edge samples, placed by a prefix sum
+            uint32_t incl = ne, total = 0;
+            if (__any_sync(0xffffffffu, ne != 0)) {      // about one element in five has none
 #pragma unroll
-                    for (int off = 1; off < 32; off <<= 1) {
-                        const uint32_t t2 = __shfl_up_sync(0xffffffffu, incl, off);
-                        if ((int)lane >= off)
-                            incl += t2;
-                    }
-                    total = __shfl_sync(0xffffffffu, incl, 31);
+                for (int off = 1; off < 32; off <<= 1) {
+                    const uint32_t t2 = __shfl_up_sync(0xffffffffu, incl, off);
+                    if ((int)lane >= off)
+                        incl += t2;
                 }
-                if (total != 0u) {
-                    int pos = queued + (int)(incl - ne);
-                    uint64_t rest = edges;
-                    while (rest) {
-                        const int q = __ffsll((long long)rest) - 1;
-                        rest &= rest - 1;
-                        wq[warp].q[pos++] = EdgeEntry{(uint32_t)(t.first + s), K == 3 ? (block << 5) | (uint32_t)q : (uint32_t)q};
-                    }
-                    queued += (int)total;
-                    drain(queued, false);
-                }
-            } else {
-                // each lane's lowest remaining edge sample per round: as many
-                // rounds as the most edge samples of any lane's fragment
+                total = __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (total != 0u) {
+                int pos = queued + (int)(incl - ne);
                 uint64_t rest = edges;
-                while (__any_sync(0xffffffffu, rest != 0)) {
-                    const bool has = rest != 0;
-                    const unsigned mask = __ballot_sync(0xffffffffu, has);
-                    if (has) {
-                        const int q = __ffsll((long long)rest) - 1;
-                        rest &= rest - 1;
-                        wq[warp].q[queued + __popc(mask & below)] = EdgeEntry{(uint32_t)(t.first + s), (uint32_t)q};
-                    }
-                    queued += __popc(mask);
-                    drain(queued, false);
+                while (rest) {
+                    const int q = __ffsll((long long)rest) - 1;
+                    rest &= rest - 1;
+                    wq[warp].q[pos++] = EdgeEntry{(uint32_t)(frag), K == 3 ? (block << 5) | (uint32_t)q : (uint32_t)q};
                 }
+                queued += (int)total;
+                drain(queued, false);
+            }
+        } else {
+            // each lane's lowest remaining edge sample per round: as many
+            // rounds as the most edge samples of any lane's fragment
+            uint64_t rest = edges;
+            while (__any_sync(0xffffffffu, rest != 0)) {
+                const bool has = rest != 0;
+                const unsigned mask = __ballot_sync(0xffffffffu, has);
+                if (has) {
+                    const int q = __ffsll((long long)rest) - 1;
+                    rest &= rest - 1;
+                    wq[warp].q[queued + __popc(mask & below)] = EdgeEntry{(uint32_t)(frag), (uint32_t)q};
+                }
+                queued += __popc(mask);
+                drain(queued, false);
             }
         }
         if (!more)
             break;
-        tile = nt;
-        t = tn;
+        strip = ns;
     }
     drain(queued, true);
 }
 
 template <int K>
-int launch_rpcf(const rbsm_map &map, const rbsm_frags &f, float *vis, int max_dist, unsigned long long *ctr,
-                cudaStream_t stream)
+int launch_rpcf(const rbsm_map &map, const rbsm_frags &f, float *vis, int max_dist, cudaStream_t stream)
 {
-    auto kern = rpcf_kernel<K, kRpcfThreads>;
+    auto kern = rpcf_kernel<K, kRpcfThreads<K>>;
     static KernelSetup setup;
     int occupancy = 0;
-    int rc = setup.get(kern, kRpcfThreads, 0, &occupancy);
+    int rc = setup.get(kern, kRpcfThreads<K>, 0, &occupancy);
     if (rc != RBSM_OK)
         return rc;
     const int sms = device_sm_count();
     if (sms <= 0)
         return cuda_fail(cudaErrorNoDevice);
-    const long long warp_tiles = (f.n + kWarpTile - 1) / kWarpTile;
-    const long long blocks_needed = (warp_tiles + kRpcfThreads / 32 - 1) / (kRpcfThreads / 32);
+    const long long strips = (f.n + 31) / 32;
+    const long long blocks_needed = (strips + kRun - 1) / kRun;
     long long grid = (long long)sms * occupancy;
     if (grid > blocks_needed)
         grid = blocks_needed;
-    const bool vec = aligned16(f.x) && aligned16(f.y) && aligned16(f.z);
-    if (K > 1 && ctr) {
-        const cudaError_t ez = cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), stream);
-        if (ez != cudaSuccess)
-            return cuda_fail(ez);
-    }
-    kern<<<(unsigned)grid, kRpcfThreads, 0, stream>>>(to_dev(map), f.x, f.y, f.z, f.n, vis, max_dist, vec,
-                                                      K > 1 ? ctr : nullptr);
+    kern<<<(unsigned)grid, kRpcfThreads<K>, 0, stream>>>(to_dev(map), f.x, f.y, f.z, f.n, vis, max_dist);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return cuda_fail(e);
@@ -447,8 +452,9 @@ int launch_rpcf(const rbsm_map &map, const rbsm_frags &f, float *vis, int max_di
 namespace rbsm {
 namespace {
 
+// ws: the caller's workspace, checked and not used (nullptr: none)
 int rpcf_entry(const rbsm_map *map, const rbsm_frags *frags, float *vis, int32_t k, const rbsm_params *params,
-               unsigned long long *ctr, void *stream)
+               const void *ws, void *stream)
 {
     int rc, max_dist;
     if ((rc = check_map(map)) != RBSM_OK) return rc;
@@ -465,16 +471,16 @@ int rpcf_entry(const rbsm_map *map, const rbsm_frags *frags, float *vis, int32_t
     // vis holds partial sums while the kernel runs: it must not overlap an input
     if (overlaps_inputs(*map, *frags, vis, (size_t)frags->n * 4u))
         return RBSM_ERR_ARG;
-    if (ctr && (overlaps_inputs(*map, *frags, ctr, 8) ||
-                (reinterpret_cast<uintptr_t>(ctr) < reinterpret_cast<uintptr_t>(vis) + (uintptr_t)frags->n * 4u &&
-                 reinterpret_cast<uintptr_t>(vis) < reinterpret_cast<uintptr_t>(ctr) + 8u)))
+    if (ws && (overlaps_inputs(*map, *frags, ws, 8) ||
+               (reinterpret_cast<uintptr_t>(ws) < reinterpret_cast<uintptr_t>(vis) + (uintptr_t)frags->n * 4u &&
+                reinterpret_cast<uintptr_t>(vis) < reinterpret_cast<uintptr_t>(ws) + 8u)))
         return RBSM_ERR_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     switch (k) {
-    case 1: return launch_rpcf<1>(*map, *frags, vis, max_dist, ctr, s);
-    case 3: return launch_rpcf<3>(*map, *frags, vis, max_dist, ctr, s);
-    case 5: return launch_rpcf<5>(*map, *frags, vis, max_dist, ctr, s);
-    default: return launch_rpcf<7>(*map, *frags, vis, max_dist, ctr, s);
+    case 1: return launch_rpcf<1>(*map, *frags, vis, max_dist, s);
+    case 3: return launch_rpcf<3>(*map, *frags, vis, max_dist, s);
+    case 5: return launch_rpcf<5>(*map, *frags, vis, max_dist, s);
+    default: return launch_rpcf<7>(*map, *frags, vis, max_dist, s);
     }
 }
 
@@ -492,5 +498,5 @@ extern "C" int rbsm_rpcf_ws(const rbsm_map *map, const rbsm_frags *frags, float 
 {
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 7u) != 0)
         return RBSM_ERR_ARG;
-    return rbsm::rpcf_entry(map, frags, vis, k, params, reinterpret_cast<unsigned long long *>(workspace), stream);
+    return rbsm::rpcf_entry(map, frags, vis, k, params, workspace, stream);
 }
