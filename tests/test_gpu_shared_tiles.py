@@ -1,0 +1,66 @@
+"""GPU test of the kernels whose CTAs share out their tiles (single-map calls,
+depth buffers, RPCF): a fragment's answer does not depend on how many
+fragments follow it, so the answers of n fragments are the first n of a larger
+call's, bit for bit, for n around the strips, runs, CTA shapes and waves the
+launches switch at; and nothing past the last fragment is written."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def scene():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1711_07793_gb300 import api
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g = torch.Generator(device="cuda").manual_seed(3)
+    depth = torch.where(torch.rand((250, 384), generator=g, device="cuda") < 0.01, 0.3, 1.0)
+    n = sms * 40 * 128 * 3 + 77
+    x, y = (torch.rand(n, generator=g, device="cuda") * 1.02 - 0.01 for _ in range(2))
+    return api, sms, depth, x, y, torch.full((n,), 0.75, device="cuda")
+
+
+def _counts(sms):
+    return [1, 31, 33, 127, 129, 257, 8 * 32 * sms + 1, 128 * 32 * sms - 127, 128 * 32 * sms + 1, 128 * 40 * sms + 129]
+
+
+@pytest.mark.parametrize("texture", [False, True])
+@pytest.mark.parametrize("what", ["silhouette", "filter", "rpcf1", "rpcf3", "rpcf5"])
+def test_a_prefix_gives_the_prefix(scene, what, texture):
+    api, sms, depth, x, y, z = scene
+    m = api.MapTexture(depth) if texture else depth
+
+    def call(n, out):
+        if what.startswith("rpcf"):
+            return api.rbsm_rpcf(m, x[:n], y[:n], z[:n], k=int(what[4:]), vis=out)
+        return (api.rbsm_visibility if what == "silhouette" else api.rsmss_filter)(m, x[:n], y[:n], z[:n], vis=out)[0]
+
+    full = call(x.numel(), torch.empty_like(x))
+    for n in _counts(sms):
+        out = torch.full((n + 40,), -7.0, device="cuda")
+        call(n, out[:n])
+        assert torch.equal(out[:n], full[:n]), n
+        assert bool((out[n:] == -7.0).all()), n
+
+
+def test_a_prefix_of_the_rows_of_a_depth_buffer(scene):
+    api, sms, depth, _, _, _ = scene
+    w = 997
+    full_h = 128 * 40 * sms * 2 // w
+    g = torch.Generator(device="cuda").manual_seed(4)
+    d = torch.rand((full_h, w), generator=g, device="cuda")
+    m = np.eye(4, dtype=np.float32)
+    m[0, 0], m[1, 1] = 1.0 / w, 1.0 / full_h
+    full = api.GBufferJob(depth, d, m)
+    api.rbsm_visibility_gbuffer([full])
+    for h in (1, 2, 40, 128 * 20 * sms // w, full_h - 1):
+        job = api.GBufferJob(depth, d[:h], m)
+        api.rbsm_visibility_gbuffer([job])
+        assert torch.equal(job.vis_silhouette, full.vis_silhouette[:h * w])
+        assert torch.equal(job.vis_filter, full.vis_filter[:h * w])
