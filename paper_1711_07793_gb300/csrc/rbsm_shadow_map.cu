@@ -3,14 +3,14 @@
 // (i + 0.5, j + 0.5) and keeps the smallest depth of the oriented
 // rectangles and sphere caps covering it.
 //
-// A CTA owns 32 x 32 texel tiles (persistent, grid-stride over tiles).  Per
-// tile it culls the occluders of both kinds, 256 at a time, with float tests
+// A CTA owns square tiles of 32 or 64 texels a side (persistent, grid-stride
+// over tiles).  Per tile it culls the occluders of both kinds, 256 at a time, with float tests
 // that can only keep too many (the tile's texel centres projected on the
 // rectangle's own two axes, the disc against the box of texel centres, both
 // widened by half a texel), gathers the survivors in shared memory in index
-// order, and every thread tests its 4 texels against them.  Double precision is slow on
-// this GPU, so the map's double-precision definition is reached mostly in
-// float:
+// order, and its warps test blocks of 32 x 4 texels against them, a column of
+// 4 per thread.  Double precision is slow on this GPU, so the map's
+// double-precision definition is reached mostly in float:
 //   * the coverage tests run first in float, relative to the tile centre,
 //     with an error bound: a decision further than the bound from its
 //     threshold is the exact one;
@@ -36,8 +36,9 @@
 namespace rbsm {
 namespace {
 
-constexpr int kTile = 32;                 // texels per tile side
-constexpr int kSmThreads = 256;           // 8 rows of 32 per pass, 4 passes
+constexpr int kSmThreads = 256;           // 8 warps
+constexpr int kLargeTile = 64;            // texels per tile side on large maps
+constexpr int kBlockRows = 4;             // a warp works on blocks of 32 x 4 texels
 constexpr int kChunk = kSmThreads;        // occluders culled per round
 constexpr float kCullSlack = 0.5f;        // texels added to every (float) culling bound
 
@@ -80,7 +81,7 @@ constexpr int kSmWarps = kSmThreads / 32;
 struct TileSmem {
     Cand c[2][kChunk];
     int idx[kChunk];                          // survivors' slots: rectangles, then spheres, in index order
-    int cnt_r[kSmWarps], cnt_s[kSmWarps];     // survivors per warp, for the order-keeping offsets
+    alignas(16) int cnt[kSmWarps];            // survivors per warp (rectangles | spheres << 16), for the order-keeping offsets
 };
 
 // Float copies of up to kFloatCopies occluders of each kind, made once per
@@ -277,7 +278,7 @@ __device__ __noinline__ float cap_depth_exact(const rbsm_sphere *cp, int i, int 
 // `fast`, the float-float data of the cap depth), each kind in index order
 // (ballots and per-warp counts, so every texel meets its occluders in the
 // definition's order).  nr, ns: the survivors of each kind.
-template <bool COPIES>
+template <bool COPIES, int kTile>
 __device__ __forceinline__ void cull_round(const rbsm_occluders &occ, const FloatOcc *fo, const FloatSph *fs,
                                            long long base, float tcx, float tcy, bool fast, TileSmem &sm,
                                            Cand *buf, int &nr, int &ns)
@@ -341,27 +342,25 @@ __device__ __forceinline__ void cull_round(const rbsm_occluders &occ, const Floa
         }
     }
     const unsigned br = __ballot_sync(0xffffffffu, keep_r), bs = __ballot_sync(0xffffffffu, keep_s);
-    if (lane == 0) {
-        sm.cnt_r[warp] = __popc(br);
-        sm.cnt_s[warp] = __popc(bs);
-    }
+    if (lane == 0)
+        sm.cnt[warp] = __popc(br) | (__popc(bs) << 16);
     __syncthreads();
-    int off_r = 0, off_s = 0;
-    nr = 0;
-    ns = 0;
+    const int4 c0 = *reinterpret_cast<const int4 *>(&sm.cnt[0]);
+    const int4 c1 = *reinterpret_cast<const int4 *>(&sm.cnt[4]);
+    const int cnt[kSmWarps] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+    int off = 0, all = 0;
 #pragma unroll
     for (int w = 0; w < kSmWarps; ++w) {
-        const int cr = sm.cnt_r[w], cs = sm.cnt_s[w];
-        off_r += w < warp ? cr : 0;
-        off_s += w < warp ? cs : 0;
-        nr += cr;
-        ns += cs;
+        off += w < warp ? cnt[w] : 0;
+        all += cnt[w];
     }
+    nr = all & 0xffff;
+    ns = all >> 16;
     const unsigned below = (1u << lane) - 1u;
     if (keep_r)
-        sm.idx[off_r + __popc(br & below)] = (int)threadIdx.x;
+        sm.idx[(off & 0xffff) + __popc(br & below)] = (int)threadIdx.x;
     if (keep_s)
-        sm.idx[nr + off_s + __popc(bs & below)] = (int)threadIdx.x;
+        sm.idx[nr + (off >> 16) + __popc(bs & below)] = (int)threadIdx.x;
     __syncthreads();
 }
 
@@ -370,7 +369,18 @@ __device__ __forceinline__ void cull_round(const rbsm_occluders &occ, const Floa
 // CTA holds float copies of all occluders (neither kind has more than
 // kFloatCopies); a compile-time choice, so that the culling holds no
 // double-to-float conversions (slow FP64 pipe) when it reads the copies.
-template <bool COPIES>
+//
+// kTile: texels per tile side, 32 (one block per warp) or a larger multiple
+// of 32 (several blocks per warp, and at most kChunk occluders in all).
+//
+// Bound: instruction issue.  Culling a tile costs a warp about 270
+// instructions whatever the tile holds, so large maps take tiles of 64 and
+// the warps turn survivors down (or take a rectangle over the whole of a
+// block) block by block: 8192^2 texels with 140 rectangles and 60 spheres,
+// 4 maps in a call, 202 us a map with tiles of 32 and 150 with 64 (96: 161,
+// 128: 160; blocks handed to the warps one at a time: 163).  One map's 268 MB
+// take 40 us at the copy rate.
+template <bool COPIES, int kTile>
 __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_occluders occ, float *__restrict__ depth,
                                                                 int width, int height, long long pitch,
                                                                 double inv_zscale)
@@ -393,103 +403,135 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
     // the float-float cap depth needs 1 / zscale exact in float
     const bool fast = inv_zscale >= 7.888609052210118e-31 && inv_zscale <= 1.2676506002282294e30;   // 2^-100, 2^100
     const float invf = (float)inv_zscale;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    // the warp's index through a shuffle: the same on all lanes for the compiler too
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
     constexpr float h = 0.5f * (kTile - 1);
-    // texel centre - tile centre, exact: ox for this thread's column, oy[p]
-    // for its rows ty + 8 p
-    const float ox = __fsub_rn(small_int_float(tx), h);
-    float oys[4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-        oys[p] = __fsub_rn(small_int_float(ty + 8 * p), h);
     const long long n_all = (long long)occ.n_rects + occ.n_spheres;
-    const long long pitch8 = pitch * 8;
     unsigned round = 0;                        // culling rounds so far (selects the candidate buffer)
     // the tile's column and row, stepped by the grid stride (no division per
-    // tile), and the offset of this thread's first row in the map
+    // tile)
     const int tiles_x = (width + kTile - 1) / kTile;
     const int tiles = tiles_x * ((height + kTile - 1) / kTile);     // <= 2^22
     int tcol = (int)blockIdx.x % tiles_x, trow = (int)blockIdx.x / tiles_x;
     const int step_col = (int)gridDim.x % tiles_x, step_row = (int)gridDim.x / tiles_x;
-    const long long tile_rows = (long long)kTile * pitch;
-    const long long step_rows = (long long)step_row * tile_rows;
-    long long row0 = (long long)trow * tile_rows + (long long)ty * pitch;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int i0 = tcol * kTile, j0 = trow * kTile;
-        float *out = depth + row0 + i0 + tx;
         tcol += step_col;
         trow += step_row;
-        row0 += step_rows;
         if (tcol >= tiles_x) {
             tcol -= tiles_x;
             ++trow;
-            row0 += tile_rows;
         }
-        // tile centre (i0 + 0.5 + 15.5, j0 + 16), exact (< 2^23)
+        // tile centre (i0 + 0.5 + (kTile - 1) / 2, ...), exact (< 2^23)
         const float tcx = small_int_float(i0 + kTile / 2), tcy = small_int_float(j0 + kTile / 2);
-        const int i = i0 + tx;
-        float best[4];
-#pragma unroll
-        for (int p = 0; p < 4; ++p)
-            best[p] = occ.ground;
-        // occluders in rounds of kChunk: rectangles, then spheres, in index
-        // order
-        for (long long base = 0; base < n_all; base += kChunk) {
-            int nr, ns;
-            Cand *buf = sm.c[round & 1];
-            ++round;
-            cull_round<COPIES>(occ, fop, fsp, base, tcx, tcy, fast, sm, buf, nr, ns);
+        // one block of 32 x 4 texels (this thread: a column of 4) against the
+        // survivors of a culling round
+        auto test_block = [&](int bi, int bj, const Cand *buf, int nr, int ns, float (&best)[kBlockRows]) {
+            // block centre and this thread's texel centres - tile centre, exact
+            const float bx = __fsub_rn(small_int_float(bi) + 15.5f, h), by = __fsub_rn(small_int_float(bj) + 1.5f, h);
+            const float ox = __fsub_rn(small_int_float(bi + lane), h), oy0 = by - 1.5f;
             for (int q = 0; q < nr; ++q) {
                 const RectCand &r = buf[sm.idx[q]].r;
+                // the block against the rectangle: |s| within 15.5 |ux| + 1.5 |uy| of its centre's
+                const float sb = fabsf(r.s0 + (bx * r.uxf + by * r.uyf)), tb = fabsf(r.t0 + (by * r.uxf - bx * r.uyf));
+                const float ss = 15.5f * fabsf(r.uxf) + 1.5f * fabsf(r.uyf) + 2.0f * r.es;
+                const float st = 15.5f * fabsf(r.uyf) + 1.5f * fabsf(r.uxf) + 2.0f * r.et;
+                if (sb > r.haf + ss || tb > r.hbf + st)
+                    continue;                              // surely outside
+                if (sb + ss < r.haf && tb + st < r.hbf) {
+#pragma unroll
+                    for (int p = 0; p < kBlockRows; ++p)   // surely covers the block
+                        best[p] = r.depth < best[p] ? r.depth : best[p];
+                    continue;
+                }
                 const float sx = ox * r.uxf, tx_ = -ox * r.uyf;
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                    const float oy = oys[p];
+                for (int p = 0; p < kBlockRows; ++p) {
+                    const float oy = oy0 + (float)p;
                     const float sf = fabsf(r.s0 + (sx + oy * r.uyf));
                     const float tf = fabsf(r.t0 + (tx_ + oy * r.uxf));
                     if (sf > r.haf + r.es || tf > r.hbf + r.et || !(r.depth < best[p]))
-                        continue;                      // surely outside, or it cannot lower the depth
+                        continue;                          // surely outside, or it cannot lower the depth
                     bool in = sf < r.haf - r.es && tf < r.hbf - r.et;
                     if (!in)
-                        in = rect_covers_exact(occ.rects + r.k, i, j0 + ty + 8 * p);     // near an edge
+                        in = rect_covers_exact(occ.rects + r.k, i0 + bi + lane, j0 + bj + p);     // near an edge
                     if (in)
                         best[p] = r.depth;
                 }
             }
             for (int q = 0; q < ns; ++q) {
                 const SphereCand &c = buf[sm.idx[nr + q]].s;
+                // the disc against the block's box of texel centres
+                const float gx = fmaxf(fabsf(c.dx0 + bx) - 15.5f, 0.0f), gy = fmaxf(fabsf(c.dy0 + by) - 1.5f, 0.0f);
+                if (gx * gx + gy * gy > c.r2f + 2.0f * c.e)
+                    continue;                              // surely outside
                 const float dxf = c.dx0 + ox;
                 const CapColumn col = cap_column(c, ox);
                 // one copy of the cap code for the 4 rows (fewer registers):
                 // the rows' depths rotate through best[0]
-                float oy = oys[0];
+                float oy = oy0;
 #pragma unroll 1
-                for (int p = 0; p < 4; ++p) {
+                for (int p = 0; p < kBlockRows; ++p) {
                     const float dyf = c.dy0 + oy;
                     // skip when it cannot lower the depth, or surely outside the disc
                     if (c.dmin < best[0] && !(dxf * dxf + dyf * dyf > c.r2f + c.e)) {
                         float d = 0.0f;
                         const int cap = c.fast ? cap_fast(c, col, oy, invf, d) : -1;
                         if (cap < 0)
-                            d = cap_depth_exact(occ.spheres + c.k, i, j0 + ty + 8 * p, inv_zscale, occ.zscale);
+                            d = cap_depth_exact(occ.spheres + c.k, i0 + bi + lane, j0 + bj + p, inv_zscale, occ.zscale);
                         if (cap != 0 && d < best[0])
                             best[0] = d;
                     }
-                    const float b = best[0];
+                    const float f = best[0];
                     best[0] = best[1];
                     best[1] = best[2];
                     best[2] = best[3];
-                    best[3] = b;
-                    oy = __fadd_rn(oy, 8.0f);              // exact
+                    best[3] = f;
+                    oy = __fadd_rn(oy, 1.0f);              // exact
                 }
             }
-        }
-        if (i < width) {
+        };
+        auto store_block = [&](int bi, int bj, const float (&best)[kBlockRows]) {
+            const int i = i0 + bi + lane, j = j0 + bj;
+            float *out = depth + (long long)j * pitch + i;
+            if (i < width) {
 #pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                if (j0 + ty + 8 * p < height)
-                    *out = best[p];
-                out += pitch8;
+                for (int p = 0; p < kBlockRows; ++p) {
+                    if (j + p < height)
+                        *out = best[p];
+                    out += pitch;
+                }
+            }
+        };
+        if (kTile == 32) {
+            // one block per warp, against the occluders in rounds of kChunk:
+            // rectangles, then spheres, in index order
+            float best[kBlockRows];
+#pragma unroll
+            for (int p = 0; p < kBlockRows; ++p)
+                best[p] = occ.ground;
+            for (long long base = 0; base < n_all; base += kChunk) {
+                int nr, ns;
+                Cand *buf = sm.c[round++ & 1];
+                cull_round<COPIES, kTile>(occ, fop, fsp, base, tcx, tcy, fast, sm, buf, nr, ns);
+                test_block(0, warp * kBlockRows, buf, nr, ns, best);
+            }
+            store_block(0, warp * kBlockRows, best);
+        } else {
+            // one round of occluders (at most kChunk), then block after block
+            int nr = 0, ns = 0;
+            Cand *buf = sm.c[round++ & 1];
+            cull_round<COPIES, kTile>(occ, fop, fsp, 0, tcx, tcy, fast, sm, buf, nr, ns);
+#pragma unroll 1
+            for (int block = warp; block < (kTile / 32) * (kTile / kBlockRows); block += kSmWarps) {
+                const int bi = (block & (kTile / 32 - 1)) * 32, bj = block / (kTile / 32) * kBlockRows;
+                float best[kBlockRows];
+#pragma unroll
+                for (int p = 0; p < kBlockRows; ++p)
+                    best[p] = occ.ground;
+                test_block(bi, bj, buf, nr, ns, best);
+                store_block(bi, bj, best);
             }
         }
     }
@@ -507,16 +549,19 @@ int launch_map(const rbsm_occluders &occ, float *depth, int width, int height, l
                cudaStream_t stream)
 {
     const bool copies = occ.n_rects <= kFloatCopies && occ.n_spheres <= kFloatCopies;
-    static KernelSetup setup_copies, setup_plain;
-    auto kern = copies ? shadow_map_kernel<true> : shadow_map_kernel<false>;
-    int occupancy = 0;
-    int rc = (copies ? setup_copies : setup_plain).get(kern, kSmThreads, 0, &occupancy);
-    if (rc != RBSM_OK)
-        return rc;
     const int sms = device_sm_count();
     if (sms <= 0)
         return cuda_fail(cudaErrorNoDevice);
-    const long long tiles = (long long)((width + kTile - 1) / kTile) * ((height + kTile - 1) / kTile);
+    auto tiles_of = [&](long long side) { return ((width + side - 1) / side) * ((height + side - 1) / side); };
+    const bool large = copies && (long long)occ.n_rects + occ.n_spheres <= kChunk && tiles_of(kLargeTile) >= 2LL * 4 * sms;
+    static KernelSetup setup[3];
+    const int which = large ? 2 : copies ? 1 : 0;
+    auto kern = large ? shadow_map_kernel<true, kLargeTile> : copies ? shadow_map_kernel<true, 32> : shadow_map_kernel<false, 32>;
+    int occupancy = 0;
+    int rc = setup[which].get(kern, kSmThreads, 0, &occupancy);
+    if (rc != RBSM_OK)
+        return rc;
+    const long long tiles = tiles_of(large ? kLargeTile : 32);
     long long grid = (long long)sms * occupancy;
     if (grid > tiles)
         grid = tiles;
