@@ -21,9 +21,8 @@
 //     result; when the float-float value is further than B from every float
 //     rounding boundary, its rounding is the double result's;
 //   * everything else (texels within the bound of an edge, the few cap
-//     depths near a rounding boundary, scales z that are not powers of two)
-//     takes the exact double operations in the defined order without
-//     contraction,
+//     depths near a rounding boundary) takes the exact double operations in
+//     the defined order without contraction,
 // so the map is bit-exact.
 #include <cuda_runtime.h>
 
@@ -194,16 +193,21 @@ __device__ __forceinline__ CapColumn cap_column(const SphereCand &c, float ox)
 //   sqrt(ah + al) ~ r0 + corr with r0 = sqrt(ah) (correctly rounded) and
 //   one Newton step, corr = (ah - r0^2 + al) / (2 r0): error at most
 //   2^-42 r0 with a reciprocal good to 2^-21, plus E_A / r0 from A.  The
-//   scale 1/z is a power of two (exact in float), so the drop is
-//   (r0 + corr)/z exactly.  v = (ch - dh) + ((vl + cl) - dl) then carries
+//   scale 1/z is held as ih + il within 2^-47.9 / z (il = 0 and no error when
+//   z is a power of two), and the drop (r0 + corr)/z as dh + dl: r0 ih is
+//   exact (FMA), corr il (at most 2^-47 of the drop D, |corr| <= 2^-23 r0) is
+//   left out, and the two additions of dl round at 1.5 2^-47 D and 2^-46 D,
+//   so the drop is within 2^-44.6 D of the one from the root held, which has
+//   2^-42 D (B takes 2^-40).  v = (ch - dh) + ((vl + cl) - dl) then carries
 //   2^-48 |c| from the split of c and 2^-22 (|vl| + |cl| + |dl|) from the
 //   two roundings.  The double operations themselves are within 2^-53 (|c|
-//   + 4 D + 8.2 R^2 / (r0 z)) of the real depth (D = the drop; rho^2 within
+//   + 5 D + 8.2 R^2 / (r0 z)) of the real depth (D = the drop; rho^2 within
 //   4 roundings, A within 6u_d R^2, then the square root, the scale and the
 //   subtraction).  B below adds all of these with a factor 2 to spare, and
 //   the test asks for 2 B of room, so the decision holds under the rounding
 //   of B's own evaluation.
-__device__ __forceinline__ int cap_fast(const SphereCand &c, const CapColumn &k, float oy, float invf, float &d)
+__device__ __forceinline__ int cap_fast(const SphereCand &c, const CapColumn &k, float oy, float invf, float invl,
+                                        float &d)
 {
     float sh, sl, dyh, dyl;
     two_sum(oy, c.dy0h, sh, sl);
@@ -222,12 +226,13 @@ __device__ __forceinline__ int cap_fast(const SphereCand &c, const CapColumn &k,
     const float r0 = __fsqrt_rn(ah);
     const float rr = __fdividef(1.0f, r0);                                 // 1 / r0 within 2 ulp
     const float corr = __fmul_rn(__fadd_rn(__fmaf_rn(-r0, r0, ah), al), __fmul_rn(0.5f, rr));
-    const float dh = __fmul_rn(r0, invf), dl = __fmul_rn(corr, invf);    // exact (power of two)
+    const float dh = __fmul_rn(r0, invf);
+    const float dl = __fmaf_rn(r0, invl, __fmaf_rn(corr, invf, __fmaf_rn(r0, invf, -dh)));
     float vh, vl, f, r;
     two_sum(c.ch, -dh, vh, vl);
     two_sum(vh, __fsub_rn(__fadd_rn(vl, c.cl), dl), f, r);               // f + r = the float-float depth
     const float B = 7.105427357601002e-15f * fabsf(c.ch)                                  // 2^-47
-                    + invf * (4.547473508864641e-13f * r0                                  // 2^-41
+                    + invf * (9.094947017729282e-13f * r0                                  // 2^-40
                               + (1.01f * ea + 8.881784197001252e-16f * c.r2h) * rr)       // 2^-50
                     + 2.384185791015625e-07f * (fabsf(vl) + fabsf(c.cl) + fabsf(dl))       // 2^-22
                     + 7.52316384526264e-37f;                                               // 2^-120
@@ -383,7 +388,7 @@ __device__ __forceinline__ void cull_round(const rbsm_occluders &occ, const Floa
 template <bool COPIES, int kTile>
 __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_occluders occ, float *__restrict__ depth,
                                                                 int width, int height, long long pitch,
-                                                                double inv_zscale)
+                                                                double inv_zscale, float scale_hi, float scale_lo)
 {
     // the next map's kernel (a programmatic dependent when the maps share no
     // memory) may take SMs as this one's CTAs finish
@@ -400,9 +405,9 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
     }
     const FloatOcc *fop = fo;
     const FloatSph *fsp = fs;
-    // the float-float cap depth needs 1 / zscale exact in float
-    const bool fast = inv_zscale >= 7.888609052210118e-31 && inv_zscale <= 1.2676506002282294e30;   // 2^-100, 2^100
-    const float invf = (float)inv_zscale;
+    // 1 / zscale for the float-float cap depth: scale_hi + scale_lo, or no
+    // float-float depths (scale_hi = 0: a scale out of its range)
+    const bool fast = scale_hi > 0.0f;
     const int lane = threadIdx.x & 31;
     // the warp's index through a shuffle: the same on all lanes for the compiler too
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
@@ -477,7 +482,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
                     // skip when it cannot lower the depth, or surely outside the disc
                     if (c.dmin < best[0] && !(dxf * dxf + dyf * dyf > c.r2f + c.e)) {
                         float d = 0.0f;
-                        const int cap = c.fast ? cap_fast(c, col, oy, invf, d) : -1;
+                        const int cap = c.fast ? cap_fast(c, col, oy, scale_hi, scale_lo, d) : -1;
                         if (cap < 0)
                             d = cap_depth_exact(occ.spheres + c.k, i0 + bi + lane, j0 + bj + p, inv_zscale, occ.zscale);
                         if (cap != 0 && d < best[0])
@@ -567,6 +572,10 @@ int launch_map(const rbsm_occluders &occ, float *depth, int width, int height, l
         grid = tiles;
     int e2 = 0;
     const double inv = std::frexp(occ.zscale, &e2) == 0.5 ? std::ldexp(1.0, 1 - e2) : 0.0;
+    // 1 / zscale as a pair of floats, for scales of 2^-100 to 2^100
+    const double inv_any = 1.0 / occ.zscale;
+    const bool fast = inv_any >= 7.888609052210118e-31 && inv_any <= 1.2676506002282294e30;
+    const float hi = fast ? (float)inv_any : 0.0f, lo = fast ? (float)(inv_any - (double)hi) : 0.0f;
     cudaError_t e;
     if (overlap) {
         cudaLaunchConfig_t cfg = {};
@@ -579,9 +588,9 @@ int launch_map(const rbsm_occluders &occ, float *depth, int width, int height, l
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, kern, occ, depth, width, height, pitch, inv);
+        e = cudaLaunchKernelEx(&cfg, kern, occ, depth, width, height, pitch, inv, hi, lo);
     } else {
-        kern<<<(unsigned)grid, kSmThreads, 0, stream>>>(occ, depth, width, height, pitch, inv);
+        kern<<<(unsigned)grid, kSmThreads, 0, stream>>>(occ, depth, width, height, pitch, inv, hi, lo);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess)
