@@ -64,3 +64,32 @@ def test_a_prefix_of_the_rows_of_a_depth_buffer(scene):
         api.rbsm_visibility_gbuffer([job])
         assert torch.equal(job.vis_silhouette, full.vis_silhouette[:h * w])
         assert torch.equal(job.vis_filter, full.vis_filter[:h * w])
+
+
+@pytest.mark.parametrize("texture", [False, True])
+@pytest.mark.parametrize("k", [3, 5, 7])
+def test_rpcf_shadow_tests_on_special_depths(scene, k, texture):
+    """RPCF takes its block's shadow tests from the signs of sums, the filter
+    from comparisons: on maps and fragments of signed zeros, subnormals,
+    infinities, NaN and equal depths it is the mean of the filter's answers at
+    the shifted positions (exact in float32 on a power-of-two map), within the
+    samples' rounding of 2^-21."""
+    api = scene[0]
+    w = 64
+    v = torch.tensor([0.0, -0.0, 1e-45, -1e-45, 1e-38, 1.0, -1.0, 3e38, float("inf"), -float("inf"), float("nan")],
+                     device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(k)
+    depth = v[torch.randint(0, len(v), (w, w), generator=g, device="cuda")].contiguous()
+    # runs of one value, so that walks go on
+    depth[8:24, 8:56], depth[30:34, 4:60], depth[40:60, 20:22] = 0.0, -0.0, float("inf")
+    n = w * w * 8
+    i = torch.randint(0, w, (2, n), generator=g, device="cuda")
+    x, y = ((t + 0.25 * (1 + (t + s) % 3)).float() / w for s, t in enumerate(i))
+    z = v[torch.randint(0, len(v), (n,), generator=g, device="cuda")]
+    m = api.MapTexture(depth) if texture else depth
+    got = api.rbsm_rpcf(m, x, y, z, k=k)
+    half, ref = (k - 1) // 2, torch.zeros(n, dtype=torch.float64, device="cuda")
+    for b in range(-half, half + 1):
+        for a in range(-half, half + 1):
+            ref += api.rsmss_filter(m, x + a / w, y + b / w, z)[0].double()
+    assert float((got.double() - ref / (k * k)).abs().max()) <= 2.0 ** -21
