@@ -96,125 +96,136 @@ struct BatchJobs {
 
 // Shared memory of the learned variant: the network's biases and weight
 // pointers and, per warp, the 32 input rows and 32 outputs of one round of
-// edge fragments.
+// edge fragments and the queue of the fragments the network may answer.
 template <int kThreads>
 struct LearnedSmem {
     mlp::InferWeights w;
     uint16_t feat[kThreads / 32][32 * mlp::kIn];
     float out[kThreads / 32][32 * mlp::kOut];
-    EdgeEntry fallback[kThreads / 32][64];      // guard-tripped fragments: < 32 left over + one round
+    EdgeEntry candidate[kThreads / 32][64];     // < 32 left over + one round
     const uint32_t *trust;                      // trusted-pattern bitmap, or nullptr (none in force)
 };
 
-// Drain rounds of up to 32 queued edge fragments with the surrogate: each
-// lane gathers its fragment's 5x5 features; the fragments whose walks stop
-// inside the window and whose pattern is trusted are packed into input rows
-// and the warp runs the network on as many m16 tiles as they fill (0, 1 or
-// 2, on the tensor cores); each of them whose error estimate is within the
-// guard takes the estimate, clamped to [0, 1]; the others (and every fragment of a job that is not in FILTER
-// mode) go to the warp's fallback queue, whose exact walks run in
-// rounds of 32 like the exact path's (walked in place, a round's few
-// fallbacks would keep most lanes idle through the walk).
+// One round of the network over up to 32 candidates (one per lane): each
+// lane gathers its fragment's 5x5 features; the fragments whose pattern is
+// trusted are packed into input rows and the warp runs the network on as many
+// m16 tiles as they fill (0, 1 or 2, on the tensor cores); each of them whose
+// error estimate is within the guard takes the estimate, clamped to [0, 1],
+// over the exact answer it has.
 template <typename Jobs, int kThreads>
-__device__ __forceinline__ void drain_queue_learned(const Jobs &jobs, WarpQueue &wq, int &count, int &fb_count,
-                                                    int max_dist, bool all, LearnedSmem<kThreads> &ls, int warp,
-                                                    float tau, unsigned long long *stats)
+__device__ __forceinline__ void network_round(const Jobs &jobs, bool valid, const EdgeEntry &q,
+                                              LearnedSmem<kThreads> &ls, int warp, float tau,
+                                              unsigned long long *stats)
 {
     const unsigned lane = lane_id();
     const unsigned below = (1u << lane) - 1u;
     const int g = lane >> 2, t = lane & 3;
     uint16_t *feat = ls.feat[warp];
     float *yout = ls.out[warp];
-    EdgeEntry *fbq = ls.fallback[warp];
-    auto drain_fallback = [&](bool every) {
-        while (fb_count >= 32 || (every && fb_count > 0)) {
-            __syncwarp();
-            const int base = fb_count >= 32 ? fb_count - 32 : 0;
-            const int k = base + (int)lane;
-            if (k < fb_count) {
-                const EdgeEntry q = fbq[k];
-                resolve_entry(jobs((int)(q.bits_job >> 8)), q, max_dist);
-            }
-            __syncwarp();
-            fb_count = base;
+    bool trusted = false;
+    uint32_t bits = 0;
+    float fx = 0.0f, fy = 0.0f, gap = 0.0f;
+    if (valid) {
+        const JobOut o = jobs((int)(q.bits_job >> 8));
+        fragment_features(o.map, __ldg(o.x + q.idx), __ldg(o.y + q.idx), __ldg(o.z + q.idx), bits, fx, fy, gap);
+        trusted = mlp::pattern_trusted(ls.trust, bits);
+    }
+    const unsigned mask = __ballot_sync(0xffffffffu, trusted);
+    const int row = __popc(mask & below);
+    if (trusted)
+        mlp::write_input_row(feat + row * mlp::kIn, bits, fx, fy, gap);
+    __syncwarp();
+    const int tiles = (__popc(mask) + 15) >> 4;          // m16 tiles with rows in use (0..2)
+    for (int mt = 0; mt < tiles; ++mt) {
+        uint32_t xa[2][4];
+        mlp::load_a(feat, mlp::kIn, mt * 16, 0, lane, xa[0]);
+        mlp::load_a(feat, mlp::kIn, mt * 16, 1, lane, xa[1]);
+        mlp::HiddenFrags h1, h2;
+        uint32_t m1, m2;
+        mlp::layer(xa, 2, ls.w.w1t, mlp::kIn, ls.w.b1, lane, h1, m1);
+        mlp::layer(h1.a, 4, ls.w.w2t, mlp::kHid, ls.w.b2, lane, h2, m2);
+        float y[4];
+        mlp::output_layer(h2, ls.w.w3t, ls.w.b3, lane, y);
+        if (t == 0) {
+            yout[(mt * 16 + g) * 2] = y[0];
+            yout[(mt * 16 + g) * 2 + 1] = y[1];
+            yout[(mt * 16 + g + 8) * 2] = y[2];
+            yout[(mt * 16 + g + 8) * 2 + 1] = y[3];
         }
-    };
+    }
+    __syncwarp();
+    bool accepted = false;
+    if (trusted) {
+        const float v = yout[row * 2], e = yout[row * 2 + 1];
+        // the network's own error estimate (a NaN never passes)
+        accepted = e <= tau && v == v;
+        if (accepted) {
+            const JobOut o = jobs((int)(q.bits_job >> 8));
+            o.fil[q.idx] = v < 0.0f ? 0.0f : (v > 1.0f ? 1.0f : v);
+            if (o.codes) {
+                const uint32_t cb = q.bits_job & 0x1fu;
+                o.codes[q.idx] = (uint16_t)((cb >> 1) | ((1u - (cb & 1u)) << 4) | (1u << 10));
+            }
+        }
+    }
+    const unsigned acc_mask = __ballot_sync(0xffffffffu, accepted);
+    if (lane == 0 && acc_mask) {
+        const unsigned long long n = (unsigned long long)__popc(acc_mask);
+        atomicAdd(&stats[0], n);
+        atomicAdd(&stats[1], 0ull - n);                  // they had been counted as fallbacks
+    }
+    __syncwarp();                                        // rows and outputs read before they are overwritten
+}
+
+// Drain rounds of up to 32 queued edge fragments of the learned variant.
+// Every fragment gets its exact answer first, in full rounds like the exact
+// path's.  The network may only answer FILTER-mode fragments whose walks stop
+// inside the 5x5 window, which the walks just told: those go to the warp's
+// candidate queue and to the network 32 at a time, and an accepted estimate
+// overwrites the exact answer.  So only the fragments that can use them pay
+// for the 25 window texels and the products, on full warps.  (The features of
+// every edge fragment first, and a second queue of walks for those turned
+// down: 128 against 97 us for one 3840x2160 frame, the same answers.)
+template <typename Jobs, int kThreads>
+__device__ __forceinline__ void drain_queue_learned(const Jobs &jobs, WarpQueue &wq, int &count, int &candidates,
+                                                    int max_dist, bool all, LearnedSmem<kThreads> &ls, int warp,
+                                                    float tau, unsigned long long *stats)
+{
+    const unsigned lane = lane_id();
+    const unsigned below = (1u << lane) - 1u;
+    EdgeEntry *cq = ls.candidate[warp];
     while (count >= 32 || (all && count > 0)) {
-        __syncwarp();
+        __syncwarp();                      // queue entries and provisional stores are visible
         const int base = count >= 32 ? count - 32 : 0;
         const int k = base + (int)lane;
-        const bool valid = k < count;
+        bool use_net = false, candidate = false;
         EdgeEntry q{0u, 0u};
-        JobOut o{};
-        if (valid) {
+        if (k < count) {
             q = wq.q[k];
-            o = jobs((int)(q.bits_job >> 8));
+            const JobOut o = jobs((int)(q.bits_job >> 8));
+            use_net = o.mode == 2;
+            const int reach = resolve_entry(o, q, max_dist);
+            candidate = use_net && (max_dist <= 2 || reach <= 2);
         }
-        const bool use_net = valid && o.mode == 2;
-        // the structural guard and the trusted-pattern bitmap need only the
-        // window pattern: fragments they turn down skip the network, and
-        // the others are packed into the first rows of the round
-        bool eligible = false;
-        uint32_t bits = 0;
-        float fx = 0.0f, fy = 0.0f, gap = 0.0f;
-        if (use_net) {
-            fragment_features(o.map, __ldg(o.x + q.idx), __ldg(o.y + q.idx), __ldg(o.z + q.idx), bits, fx, fy, gap);
-            eligible = walks_inside_window(bits, max_dist) && mlp::pattern_trusted(ls.trust, bits);
-        }
-        const unsigned elig_mask = __ballot_sync(0xffffffffu, eligible);
-        const int row = __popc(elig_mask & below);
-        if (eligible)
-            mlp::write_input_row(feat + row * mlp::kIn, bits, fx, fy, gap);
-        __syncwarp();
-        const int tiles = (__popc(elig_mask) + 15) >> 4;     // m16 tiles with rows in use (0..2)
-        for (int mt = 0; mt < tiles; ++mt) {
-            uint32_t xa[2][4];
-            mlp::load_a(feat, mlp::kIn, mt * 16, 0, lane, xa[0]);
-            mlp::load_a(feat, mlp::kIn, mt * 16, 1, lane, xa[1]);
-            mlp::HiddenFrags h1, h2;
-            uint32_t m1, m2;
-            mlp::layer(xa, 2, ls.w.w1t, mlp::kIn, ls.w.b1, lane, h1, m1);
-            mlp::layer(h1.a, 4, ls.w.w2t, mlp::kHid, ls.w.b2, lane, h2, m2);
-            float y[4];
-            mlp::output_layer(h2, ls.w.w3t, ls.w.b3, lane, y);
-            if (t == 0) {
-                yout[(mt * 16 + g) * 2] = y[0];
-                yout[(mt * 16 + g) * 2 + 1] = y[1];
-                yout[(mt * 16 + g + 8) * 2] = y[2];
-                yout[(mt * 16 + g + 8) * 2 + 1] = y[3];
-            }
-        }
-        __syncwarp();
-        bool accepted = false;
-        if (eligible) {
-            const float v = yout[row * 2], e = yout[row * 2 + 1];
-            // the network's own error estimate (a NaN never passes)
-            accepted = e <= tau && v == v;
-            if (accepted) {
-                const float vc = v < 0.0f ? 0.0f : (v > 1.0f ? 1.0f : v);
-                o.fil[q.idx] = vc;
-                if (o.codes) {
-                    const uint32_t cb = q.bits_job & 0x1fu;
-                    o.codes[q.idx] = (uint16_t)((cb >> 1) | ((1u - (cb & 1u)) << 4) | (1u << 10));
-                }
-            }
-        }
-        const bool walk = valid && !accepted;
-        const unsigned walk_mask = __ballot_sync(0xffffffffu, walk);
-        if (walk)
-            fbq[fb_count + __popc(walk_mask & below)] = q;
-        const unsigned acc_mask = __ballot_sync(0xffffffffu, accepted);
-        const unsigned fb_mask = __ballot_sync(0xffffffffu, use_net && !accepted);
-        if (lane == 0 && (acc_mask | fb_mask)) {
-            atomicAdd(&stats[0], (unsigned long long)__popc(acc_mask));
-            atomicAdd(&stats[1], (unsigned long long)__popc(fb_mask));
-        }
-        __syncwarp();
-        fb_count += __popc(walk_mask);
+        const unsigned net_mask = __ballot_sync(0xffffffffu, use_net);
+        const unsigned mask = __ballot_sync(0xffffffffu, candidate);
+        if (candidate)
+            cq[candidates + __popc(mask & below)] = q;
+        if (lane == 0 && net_mask)
+            atomicAdd(&stats[1], (unsigned long long)__popc(net_mask));
+        candidates += __popc(mask);
         count = base;
-        drain_fallback(false);
+        __syncwarp();                      // candidates written and entries read; exact answers before estimates
+        if (candidates >= 32) {
+            candidates -= 32;
+            network_round<Jobs, kThreads>(jobs, true, cq[candidates + (int)lane], ls, warp, tau, stats);
+        }
     }
-    drain_fallback(all);
+    if (all && candidates > 0) {
+        const EdgeEntry q = cq[min((int)lane, candidates - 1)];
+        network_round<Jobs, kThreads>(jobs, (int)lane < candidates, q, ls, warp, tau, stats);
+        candidates = 0;
+    }
 }
 
 template <int kThreads, bool LEARNED>
@@ -317,7 +328,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) batch_kernel(const __gri
     constexpr bool kCopyMap = kMinBlocks >= 5;
     MapDev map = a.maps[a.jobs[job].map];
     int queued = 0;
-    int fb_queued = 0;                         // learned variant: guard-tripped fragments waiting to walk
+    int candidates = 0;                        // learned variant: fragments waiting for the network
     for (;;) {
         long long nt;
         if (in_chunk + 1 < csz) {
@@ -384,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) batch_kernel(const __gri
             classify_warp_tile<kFixedMode ? kFixedMode : 1, kFixedCodes>(kCopyMap ? map : a.maps[J.map], t, c, wq,
                                                                          queued);
         if (LEARNED)
-            drain_queue_learned<BatchJobs, kThreads>(jobs, wq, queued, fb_queued, a.max_dist, false, ls, warp, a.tau,
+            drain_queue_learned<BatchJobs, kThreads>(jobs, wq, queued, candidates, a.max_dist, false, ls, warp, a.tau,
                                                      a.stats);
         else
             drain_queue<BatchJobs, kFixedMode>(jobs, wq, queued, a.max_dist, false);
@@ -397,7 +408,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) batch_kernel(const __gri
         t = tn;
     }
     if (LEARNED)
-        drain_queue_learned<BatchJobs, kThreads>(jobs, wq, queued, fb_queued, a.max_dist, true, ls, warp, a.tau,
+        drain_queue_learned<BatchJobs, kThreads>(jobs, wq, queued, candidates, a.max_dist, true, ls, warp, a.tau,
                                                  a.stats);
     else
         drain_queue<BatchJobs, kFixedMode>(jobs, wq, queued, a.max_dist, true);

@@ -124,7 +124,9 @@ __device__ __forceinline__ EdgeWalk edge_walk(const MapDev &m, const float *p, i
 
 // Walk results of the fragment at texel (i, j): rxn, rxp along x towards
 // lower and higher columns, ryn, ryp along y towards lower and higher rows.
-__device__ __forceinline__ void edge_walks(const MapDev &m, int i, int j, float pz, bool lit, unsigned d4,
+// Returns the step at which the last of the four ends (max_dist + 1 when one
+// does not).
+__device__ __forceinline__ int edge_walks(const MapDev &m, int i, int j, float pz, bool lit, unsigned d4,
                                            int max_dist, int &rxn, int &rxp, int &ryn, int &ryp)
 {
     const unsigned open = (((d4 & 12u) ? 3u : 0u) | ((d4 & 3u) ? 12u : 0u)) & ~d4;
@@ -171,6 +173,7 @@ __device__ __forceinline__ void edge_walks(const MapDev &m, int i, int j, float 
     rxp = lo == 2u ? ra : hi == 2u ? rb : (d4 & 2u) ? 1 : -1;
     ryp = lo == 4u ? ra : hi == 4u ? rb : (d4 & 4u) ? 1 : -1;
     ryn = lo == 8u ? ra : hi == 8u ? rb : (d4 & 8u) ? 1 : -1;
+    return max(lo ? abs(ra) : 1, hi ? abs(rb) : 1);
 }
 
 // Eq. 5 and the normalisation along one axis: the position of the fragment
@@ -282,11 +285,12 @@ __device__ __forceinline__ bool walks_inside_window(uint32_t pattern, int max_di
            !(goes_on_y(1) && goes_on_y(2)) && !(goes_on_y(-1) && goes_on_y(-2));
 }
 
-// Result of one fragment.
+// Result of one fragment (reach: the step its longest walk stopped at).
 struct FragResult {
     float sil;
     float fil;
     uint16_t code;
+    int reach = 0;
 };
 
 // Steps 1-2 from the five depths of the texel and its neighbours.
@@ -394,7 +398,7 @@ __device__ __forceinline__ void resolve_edge_uv(const MapDev &m, float u, float 
     const unsigned d4 = (bits >> 1) & 15u;
     // computeFragmentDistanceToSE: the four walks -x, +x, -y, +y
     int rxn, rxp, ryn, ryp;
-    edge_walks(m, i, j, pz, s0 != 0, d4, max_dist, rxn, rxp, ryn, ryp);
+    r.reach = edge_walks(m, i, j, pz, s0 != 0, d4, max_dist, rxn, rxp, ryn, ryp);
     int ex = (rxn > 0) + (rxp > 0);
     int ey = (ryn > 0) + (ryp > 0);
     float nx = axis_position(rxn, rxp, fx);
@@ -533,8 +537,9 @@ __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 // Walk, normalise and answer one deferred edge fragment; write its answers.
 // FIXED_MODE 1..3 when every job of the launch has that mode, 0 to read it
 // from the job.
+// Returns the step its longest walk stopped at.
 template <int FIXED_MODE = 0>
-__device__ __forceinline__ void resolve_entry(const JobOut &o, const EdgeEntry &q, int max_dist)
+__device__ __forceinline__ int resolve_entry(const JobOut &o, const EdgeEntry &q, int max_dist)
 {
     const uint32_t bits = q.bits_job & 0x1fu;
     const uint32_t d4 = bits >> 1, s0 = bits & 1u;
@@ -548,6 +553,7 @@ __device__ __forceinline__ void resolve_entry(const JobOut &o, const EdgeEntry &
     if (o.mode & 1) o.sil[q.idx] = r.sil;
     if (o.mode & 2) o.fil[q.idx] = r.fil;
     if (o.codes) o.codes[q.idx] = r.code;
+    return r.reach;
 }
 
 // Drain full rounds of 32 queued edge fragments (or everything when
