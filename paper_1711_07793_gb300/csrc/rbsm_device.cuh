@@ -88,9 +88,14 @@ __device__ __forceinline__ void texel_coord(float x, int size, int &t, float &f)
 // is read exists.  A walk that reaches the border stays on its texel (clamp
 // to edge), which continues the edge, for the steps that are left: it finds
 // no end, so it is stopped there.  The loads of a step, of both walks, are in
-// flight before the first test.  Loads of later steps are not issued ahead: the extra, mostly wasted,
-// requests cost more than the latency they hide (two steps per iteration
-// with their loads together: 67.2 against 60.7 us on one 3840x2160 frame).
+// flight before the first test.  Loads of later steps are not issued ahead
+// while most walks are still on: the extra, mostly wasted, requests cost more
+// than the latency they hide (two steps per iteration with their loads
+// together: 67.2 against 60.7 us on one 3840x2160 frame).  With PAIRS the
+// steps after the second, which few walks reach but those take many of, go
+// two at a time: silhouette, 1920x1080, 22.1 -> 20.1 us, filtering, 3840x2160,
+// 52.5 -> 51.8 in the single-map kernel at 64 registers; the kernels at 48
+// spill with it (cascades 369 -> 380 us) and take single steps.
 //
 // Bound: the latency of the steps and the issue slots of a round's longest
 // walk.  rsmss_filter, 3840x2160 fragments on a 4096^2 map, 5 % of them on
@@ -126,6 +131,7 @@ __device__ __forceinline__ EdgeWalk edge_walk(const MapDev &m, const float *p, i
 // lower and higher columns, ryn, ryp along y towards lower and higher rows.
 // Returns the step at which the last of the four ends (max_dist + 1 when one
 // does not).
+template <bool PAIRS>
 __device__ __forceinline__ int edge_walks(const MapDev &m, int i, int j, float pz, bool lit, unsigned d4,
                                            int max_dist, int &rxn, int &rxp, int &ryn, int &ryp)
 {
@@ -140,16 +146,8 @@ __device__ __forceinline__ int edge_walks(const MapDev &m, int i, int j, float p
     if (hi == 0u)
         B.last = 0;
     int ra = -(max_dist + 1), rb = ra;
-    for (int k = 1;; ++k) {
-        const bool a = k <= A.last, b = k <= B.last;
-        if (!a && !b)
-            break;
-        A.p += A.step;
-        B.p += B.step;
-        const float la = a ? __ldg(A.p) : 0.0f;
-        const float lb = b ? __ldg(B.p) : 0.0f;
-        const float sa = a ? __ldg(A.p + A.side) : 0.0f;
-        const float sb = b ? __ldg(B.p + B.side) : 0.0f;
+    // step k of both walks from the texels and side texels read for it
+    auto test = [&](int k, bool a, bool b, float la, float lb, float sa, float sb) {
         // a texel's test differs from the fragment's: the walk's texel (the
         // walk ends), its side texel (the walk continues the edge)
         const bool ea = (pz > la) == lit, eb = (pz > lb) == lit;
@@ -168,6 +166,33 @@ __device__ __forceinline__ int edge_walks(const MapDev &m, int i, int j, float p
             rb = eb ? k : -k;
             B.last = 0;
         }
+    };
+    int k = 1;
+    for (; !PAIRS || k <= 2; ++k) {
+        const bool a = k <= A.last, b = k <= B.last;
+        if (!a && !b)
+            break;
+        A.p += A.step;
+        B.p += B.step;
+        const float la = a ? __ldg(A.p) : 0.0f;
+        const float lb = b ? __ldg(B.p) : 0.0f;
+        const float sa = a ? __ldg(A.p + A.side) : 0.0f;
+        const float sb = b ? __ldg(B.p + B.side) : 0.0f;
+        test(k, a, b, la, lb, sa, sb);
+    }
+    for (; PAIRS && (k <= A.last || k <= B.last); k += 2) {
+        const float *pa = A.p + A.step, *pb = B.p + B.step;
+        const bool a1 = k <= A.last, b1 = k <= B.last, a2 = k < A.last, b2 = k < B.last;
+        const float la1 = a1 ? __ldg(pa) : 0.0f, sa1 = a1 ? __ldg(pa + A.side) : 0.0f;
+        const float lb1 = b1 ? __ldg(pb) : 0.0f, sb1 = b1 ? __ldg(pb + B.side) : 0.0f;
+        const float la2 = a2 ? __ldg(pa + A.step) : 0.0f, sa2 = a2 ? __ldg(pa + A.step + A.side) : 0.0f;
+        const float lb2 = b2 ? __ldg(pb + B.step) : 0.0f, sb2 = b2 ? __ldg(pb + B.step + B.side) : 0.0f;
+        A.p = pa;
+        B.p = pb;
+        test(k, a1, b1, la1, lb1, sa1, sb1);
+        A.p += A.step;
+        B.p += B.step;
+        test(k + 1, k + 1 <= A.last, k + 1 <= B.last, la2, lb2, sa2, sb2);
     }
     rxn = lo == 1u ? ra : (d4 & 1u) ? 1 : -1;
     rxp = lo == 2u ? ra : hi == 2u ? rb : (d4 & 2u) ? 1 : -1;
@@ -386,7 +411,7 @@ __device__ __forceinline__ bool classify(const MapDev &m, float x, float y, floa
 
 // Steps 3-4 for one edge fragment at texel-space position (u, v)
 // (recomputes its texel).
-template <int MODE>
+template <int MODE, bool PAIRS = false>
 __device__ __forceinline__ void resolve_edge_uv(const MapDev &m, float u, float v, float pz,
                                                 uint32_t bits, int max_dist, FragResult &r)
 {
@@ -398,7 +423,7 @@ __device__ __forceinline__ void resolve_edge_uv(const MapDev &m, float u, float 
     const unsigned d4 = (bits >> 1) & 15u;
     // computeFragmentDistanceToSE: the four walks -x, +x, -y, +y
     int rxn, rxp, ryn, ryp;
-    r.reach = edge_walks(m, i, j, pz, s0 != 0, d4, max_dist, rxn, rxp, ryn, ryp);
+    r.reach = edge_walks<PAIRS>(m, i, j, pz, s0 != 0, d4, max_dist, rxn, rxp, ryn, ryp);
     int ex = (rxn > 0) + (rxp > 0);
     int ey = (ryn > 0) + (ryp > 0);
     float nx = axis_position(rxn, rxp, fx);
@@ -412,11 +437,11 @@ __device__ __forceinline__ void resolve_edge_uv(const MapDev &m, float u, float 
 }
 
 // Steps 3-4 from a texture coordinate.
-template <int MODE>
+template <int MODE, bool PAIRS = false>
 __device__ __forceinline__ void resolve_edge(const MapDev &m, float x, float y, float pz,
                                              uint32_t bits, int max_dist, FragResult &r)
 {
-    resolve_edge_uv<MODE>(m, __fmul_rn(x, (float)m.width), __fmul_rn(y, (float)m.height), pz, bits, max_dist, r);
+    resolve_edge_uv<MODE, PAIRS>(m, __fmul_rn(x, (float)m.width), __fmul_rn(y, (float)m.height), pz, bits, max_dist, r);
 }
 
 // ------------------------------------------------------------ warp tiles --
@@ -538,7 +563,7 @@ __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 // FIXED_MODE 1..3 when every job of the launch has that mode, 0 to read it
 // from the job.
 // Returns the step its longest walk stopped at.
-template <int FIXED_MODE = 0>
+template <int FIXED_MODE = 0, bool PAIRS = false>
 __device__ __forceinline__ int resolve_entry(const JobOut &o, const EdgeEntry &q, int max_dist)
 {
     const uint32_t bits = q.bits_job & 0x1fu;
@@ -546,9 +571,9 @@ __device__ __forceinline__ int resolve_entry(const JobOut &o, const EdgeEntry &q
     FragResult r{0.0f, 0.0f, (uint16_t)(d4 | ((1u - s0) << 4))};
     const float x = __ldg(o.x + q.idx), y = __ldg(o.y + q.idx), z = __ldg(o.z + q.idx);
     switch (FIXED_MODE ? FIXED_MODE : o.mode) {
-    case 1: resolve_edge<1>(o.map, x, y, z, bits, max_dist, r); break;
-    case 2: resolve_edge<2>(o.map, x, y, z, bits, max_dist, r); break;
-    default: resolve_edge<3>(o.map, x, y, z, bits, max_dist, r); break;
+    case 1: resolve_edge<1, PAIRS>(o.map, x, y, z, bits, max_dist, r); break;
+    case 2: resolve_edge<2, PAIRS>(o.map, x, y, z, bits, max_dist, r); break;
+    default: resolve_edge<3, PAIRS>(o.map, x, y, z, bits, max_dist, r); break;
     }
     if (o.mode & 1) o.sil[q.idx] = r.sil;
     if (o.mode & 2) o.fil[q.idx] = r.fil;
@@ -559,7 +584,7 @@ __device__ __forceinline__ int resolve_entry(const JobOut &o, const EdgeEntry &q
 // Drain full rounds of 32 queued edge fragments (or everything when
 // `all`).  `jobs(job)` returns the JobOut of a job.  The count is uniform
 // across the warp.
-template <typename Jobs, int FIXED_MODE = 0>
+template <typename Jobs, int FIXED_MODE = 0, bool PAIRS = false>
 __device__ __forceinline__ void drain_queue(const Jobs &jobs, WarpQueue &wq, int &count, int max_dist, bool all)
 {
     const unsigned lane = lane_id();
@@ -569,7 +594,7 @@ __device__ __forceinline__ void drain_queue(const Jobs &jobs, WarpQueue &wq, int
         const int k = base + (int)lane;
         if (k < count) {
             const EdgeEntry q = wq.q[k];
-            resolve_entry<FIXED_MODE>(jobs((int)(q.bits_job >> 8)), q, max_dist);
+            resolve_entry<FIXED_MODE, PAIRS>(jobs((int)(q.bits_job >> 8)), q, max_dist);
         }
         __syncwarp();                      // entries read before they are overwritten
         count = base;

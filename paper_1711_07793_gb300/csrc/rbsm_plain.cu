@@ -84,7 +84,7 @@ struct PlainJobs {
 };
 
 // Persistent warps over the warp tiles of one fragment set.  A CTA owns every
-// gridDim.x-th run of kWarps consecutive tiles, so the tiles in flight gather
+// gridDim.x-th run of kRun consecutive tiles, so the tiles in flight gather
 // from one compact region of the shadow map, and its warps take them one at a
 // time from a counter in shared memory: a tile along a shadow edge drains
 // several rounds of walks (4 us each) and holds up one warp while the others
@@ -98,6 +98,11 @@ plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restric
              float *__restrict__ fil, uint16_t *__restrict__ codes, int max_dist, bool vec_planes)
 {
     constexpr int kWarps = kThreads / 32;
+    // runs of 16 tiles share the frame out more evenly than runs of a CTA's
+    // 32 (filtering 3840x2160 / 2560x1440, silhouette 1920x1080 / 1277x719
+    // unaligned: 51.5 / 33.2 / 19.8 / 20.6 us with 32, 49.2 / 31.8 / 20.2 /
+    // 18.9 with 16, 50.3 / 31.0 / 19.9 / 20.0 with 4)
+    constexpr unsigned kRun = kWarps < 16 ? kWarps : 16;
     __shared__ WarpQueue wq[kWarps];
     __shared__ float4 next[kWarps][3][32];
     __shared__ unsigned taken;                 // tiles of this CTA taken
@@ -110,7 +115,7 @@ plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restric
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
     const long long tiles = (n + kWarpTile - 1) / kWarpTile;
     auto tile_of = [&](unsigned k) {
-        return ((long long)(k / kWarps) * gridDim.x + blockIdx.x) * kWarps + k % kWarps;
+        return ((long long)(k / kRun) * gridDim.x + blockIdx.x) * kRun + k % kRun;
     };
     long long tile = tile_of((unsigned)warp);
     if (tile >= tiles)
@@ -144,20 +149,21 @@ plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restric
             stage_tile(tn, lane, buf);     // next tile's copies fly during this tile
         }
         classify_warp_tile<MODE, CODES>(m, t, c, wq[warp], queued);
-        drain_queue(jobs, wq[warp], queued, max_dist, false);
+        drain_queue<PlainJobs, MODE, kThreads == 1024>(jobs, wq[warp], queued, max_dist, false);
         if (!more)
             break;
         tile = nt;
         t = tn;
     }
-    drain_queue(jobs, wq[warp], queued, max_dist, true);
+    drain_queue<PlainJobs, MODE, kThreads == 1024>(jobs, wq[warp], queued, max_dist, true);
 }
 
 // CTAs of 1024 threads (one per SM: 32 warps share the tiles out) where the
 // tiles give every SM's 32 warps one, else of 256, which put a small launch on
 // more SMs.  3840x2160 filtering / 1920x1080 silhouette: 52.5 / 22.4 us with
 // 1024, 53.1 / 23.0 with two of 640, 52.2 / 24.4 with four of 320, 54.3 / 23.3
-// with five of 256.
+// with five of 256 (before the walks' pairs of steps and the runs of 16:
+// 49.2 / 20.2 now).
 template <int MODE, bool CODES, int kThreads>
 int launch_plain(const rbsm_map &map, const rbsm_frags &f, float *sil, float *fil, uint16_t *codes,
                  int max_dist, int sms, cudaStream_t stream)
