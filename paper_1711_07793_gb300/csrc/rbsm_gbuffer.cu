@@ -96,16 +96,19 @@ gbuffer_kernel(const MapDev m, const GBufDev g, float *__restrict__ sil, float *
         t.vec = vec_planes && t.count == kWarpTile;
         return t;
     };
-    // the depths of a tile: lane l holds fragments 4l..4l+3 (vector path,
-    // contiguous rows) or l, l+32, l+64, l+96
+    // the depths of a tile (vector path: contiguous rows)
     auto load = [&](const WarpTileIO &t, float (&d)[kPerThread]) {
         if (t.vec) {
-            const float4 v = __ldcs(reinterpret_cast<const float4 *>(g.d + t.first) + lane);
-            d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 v = __ldcs(reinterpret_cast<const float2 *>(g.d + t.first + tile_slot(true, lane, 2 * h)));
+                d[2 * h] = v.x;
+                d[2 * h + 1] = v.y;
+            }
         } else {
 #pragma unroll
             for (int e = 0; e < kPerThread; ++e) {
-                const long long f = t.first + lane + 32 * e;
+                const long long f = t.first + tile_slot(false, lane, e);
                 d[e] = 0.0f;
                 if (f < n) {
                     int px, py;
@@ -155,20 +158,20 @@ gbuffer_kernel(const MapDev m, const GBufDev g, float *__restrict__ sil, float *
             load(tn, dn);                  // next tile's loads fly during this tile
         }
         LaneCoords c;
-        // the vector path's 4 fragments are consecutive pixels: one division
-        // for the first, then steps along the row (one wrap at most when the
-        // buffer is at least 4 pixels wide)
-        const bool steps = t.vec && g.width >= kPerThread;
+        // the vector path's two pairs of pixels: one division for the first
+        // pixel, then steps of 1 and 63 along the row (one wrap at most in a
+        // buffer at least 64 pixels wide)
+        const bool steps = t.vec && g.width >= 64;
         int px = 0, py = 0;
         if (steps)
-            pixel_of(g, t.first + 4 * (long long)lane, px, py);
+            pixel_of(g, t.first + tile_slot(true, lane, 0), px, py);
 #pragma unroll
         for (int e = 0; e < kPerThread; ++e) {
-            const long long f = t.first + (t.vec ? 4 * (long long)lane + e : (long long)lane + 32 * e);
+            const long long f = t.first + tile_slot(t.vec, lane, e);
             c.x[e] = c.y[e] = c.z[e] = 0.0f;
             if (steps) {
-                if (e > 0 && ++px == g.width) {
-                    px = 0;
+                if (e > 0 && (px += e == 2 ? 63 : 1) >= g.width) {
+                    px -= g.width;
                     ++py;
                 }
                 project(g.m, px, py, d[e], c.x[e], c.y[e], c.z[e]);
