@@ -41,27 +41,28 @@ constexpr int kBlockRows = 4;             // a warp works on blocks of 32 x 4 te
 constexpr int kChunk = kSmThreads;        // occluders culled per round
 constexpr float kCullSlack = 0.5f;        // texels added to every (float) culling bound
 
-// A surviving occluder of the current tile.  Besides the exact parameters
-// (for the double-precision test) it carries its position relative to the
-// tile centre in float and an error bound E for the float pre-test: every
-// float decision further than E from its threshold is the exact one.
+// A surviving occluder of the current tile: its position relative to the tile
+// centre in float and thresholds that carry an error bound E for the float
+// tests: a float decision further than E from the true threshold is the exact
+// one.  What depends on the candidate alone is formed here, once per tile.
 struct RectCand {
-    float s0, t0, uxf, uyf, haf, hbf, es, et;   // s, t at the tile centre; bounds of the float s, t
+    float s0, t0, uxf, uyf;                       // s, t at the tile centre
+    float s_out, s_in, t_out, t_in;               // a texel is surely outside above _out, surely inside below _in
+    float bs_out, bs_in, bt_out, bt_in;           // a block's centre: surely all outside, surely all inside
     float depth;
     int k;                                        // the rectangle (its double parameters for the exact test)
 };
 
 struct SphereCand {
-    float dx0, dy0, r2f, e;                       // centre offset from the tile centre; rho^2 bound
+    float dx0, dy0, r_out, rb_out;                // centre offset; rho^2 above which a texel, a block is surely outside
     float dmin;                                   // no texel of the cap is nearer the light than this
     // float-float data of the cap depth: tile centre - disc centre
     // (dx0h + dx0l, dy0h + dy0l; within 2^-47 (|offset| + |centre|)),
     // R^2 = r2h + r2l and c = ch + cl (within 2^-47 of the doubles), the
-    // centre's magnitude (cxa, cya); fast = 0 keeps every texel on the
-    // double operations
-    float dx0h, dx0l, dy0h, dy0l, r2h, r2l, ch, cl, cxa, cya;
-    int fast;
-    int k;                                        // the sphere (its double parameters for the exact depth)
+    // centre's magnitude (cxa, cya), and the bound's share of c
+    float dx0h, dx0l, dy0h, dy0l, r2h, r2l, ch, cl, cxa, cya, b0;
+    int k;                                        // the sphere (its double parameters for the exact depth); ~k keeps
+                                                  // every texel on the double operations
 };
 
 // The survivors of one culling round (at most kChunk of both kinds): the
@@ -130,7 +131,8 @@ __device__ __forceinline__ FloatSph float_sphere(const rbsm_sphere &c, double zs
     f.r2l = (float)fma(c.radius, c.radius, -(double)f.r2h);
     f.ch = (float)c.centre_depth;
     f.cl = (float)(c.centre_depth - (double)f.ch);
-    f.fast = f.r2h >= 1e-30f && f.r2h <= 1e30f && fabsf(f.ch) <= 1e30f;
+    // (R^2 of at least 2^-66, so that every ah above 4 E_A is a normal float)
+    f.fast = f.r2h >= 1.3552527156068805e-20f && f.r2h <= 1e30f && fabsf(f.ch) <= 1e30f;
     return f;
 }
 
@@ -150,6 +152,32 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
+// The same for |a| >= |b| or a = 0 (Dekker's FastTwoSum).
+__device__ __forceinline__ void fast_two_sum(float a, float b, float &s, float &e)
+{
+    s = __fadd_rn(a, b);
+    e = __fsub_rn(b, __fsub_rn(s, a));
+}
+
+// Offset of a texel from the disc centre, o + (h + l) as a float pair: o is
+// the texel's offset from the tile centre (a multiple of 1/2, exact, at most
+// 31.5), |l| at most half an ulp of h.  Their sum s + e (TwoSum) has s = 0 or
+// |s| >= ulp(h) >= 2 |l| (or |h| >= 2^23 and s about h), and |e| <= 2^-24 |s|,
+// so FastTwoSum of s and e + l is exact.
+__device__ __forceinline__ void offset_pair(float o, float h, float l, float &dh, float &dl)
+{
+    float s, e;
+    two_sum(o, h, s, e);
+    fast_two_sum(s, __fadd_rn(e, l), dh, dl);
+}
+
+__device__ __forceinline__ float rsqrt_approx(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));       // within 2^-22.9, normal x
+    return y;
+}
+
 // The terms of R^2 - dx^2 that depend on the texel column only.
 struct CapColumn {
     float s1;      // r2h - px, high part (TwoSum)
@@ -159,17 +187,14 @@ struct CapColumn {
 
 __device__ __forceinline__ CapColumn cap_column(const SphereCand &c, float ox)
 {
-    // dx = ox + (dx0h + dx0l) as dxh + dxl (ox is exact, within 15.5)
-    float sh, sl, dxh, dxl;
-    two_sum(ox, c.dx0h, sh, sl);
-    two_sum(sh, __fadd_rn(sl, c.dx0l), dxh, dxl);
+    float dxh, dxl;
+    offset_pair(ox, c.dx0h, c.dx0l, dxh, dxl);
     const float px = __fmul_rn(dxh, dxh);
     const float pxe = __fmaf_rn(dxh, dxh, -px);                   // dxh^2 - px, exact
-    const float cxt = __fmul_rn(__fmul_rn(2.0f, dxh), dxl);       // 2 dxh dxl
     CapColumn k;
     float e1;
     two_sum(c.r2h, -px, k.s1, e1);
-    k.low = __fsub_rn(__fsub_rn(__fadd_rn(e1, c.r2l), pxe), cxt);
+    k.low = __fsub_rn(__fadd_rn(e1, c.r2l), __fmaf_rn(2.0f * dxh, dxl, pxe));
     const float mx = fabsf(ox) + fabsf(c.dx0h);
     k.ex = c.r2h + px + mx * (mx + c.cxa);
     return k;
@@ -187,18 +212,22 @@ __device__ __forceinline__ CapColumn cap_column(const SphereCand &c, float ox)
 //   2^-45 (mx + |cx|) (so dx^2 within 2^-44 mx (mx + |cx|)), the squares are
 //   exact (FMA) up to the 2 dxh dxl term (2^-47 dx^2) and the dropped dxl^2
 //   (2^-48 dx^2), and the seven low terms are summed with error at most 6u
-//   times their magnitudes (2^-43.1 of the squares).  When ah > 4 E_A and ah > 2^-40
-//   R^2, A > 2^-41 R^2, far above the 5 * 2^-53 R^2 that the double
-//   operations can move rho^2 <= R^2, so they find the texel covered.
-//   sqrt(ah + al) ~ r0 + corr with r0 = sqrt(ah) (correctly rounded) and
-//   one Newton step, corr = (ah - r0^2 + al) / (2 r0): error at most
-//   2^-42 r0 with a reciprocal good to 2^-21, plus E_A / r0 from A.  The
+//   times their magnitudes (2^-43.1 of the squares).  When ah > 4 E_A (at
+//   least 2^-39 R^2), A > 2^-40 R^2, far above the 5 * 2^-53 R^2 that the
+//   double operations can move rho^2 <= R^2, so they find the texel covered;
+//   below -6 E_A they find it outside.
+//   sqrt(ah + al) ~ r0 + corr with y = 1 / sqrt(ah) within 2^-22.9, r0 = ah y
+//   (within 2^-22.4) and one Newton step, corr = (ah - r0^2 + al) y / 2: the
+//   step leaves corr^2 / (2 r0) = 2^-44.8 r0, y stands for 1 / r0 within
+//   2^-21.7 of corr (2^-44 r0), and the three roundings of corr give 2^-46.4,
+//   2^-46.3 and 2^-46.3 r0: 2^-42.8 r0 in all, plus E_A / r0 from A.  The
 //   scale 1/z is held as ih + il within 2^-47.9 / z (il = 0 and no error when
 //   z is a power of two), and the drop (r0 + corr)/z as dh + dl: r0 ih is
-//   exact (FMA), corr il (at most 2^-47 of the drop D, |corr| <= 2^-23 r0) is
-//   left out, and the two additions of dl round at 1.5 2^-47 D and 2^-46 D,
-//   so the drop is within 2^-44.6 D of the one from the root held, which has
-//   2^-42 D (B takes 2^-40).  v = (ch - dh) + ((vl + cl) - dl) then carries
+//   exact (FMA), corr il (at most 2^-45.9 of the drop D, |corr| <= 2^-21.9 r0)
+//   is left out, and the two additions of dl round at 2^-45.6 D and 2^-45.3
+//   D, so the drop is within 2^-43.9 D of the one from the root held and
+//   2^-42.2 D of the real one (B takes 2^-40).  v = (ch - dh) + ((vl + cl) -
+//   dl) then carries
 //   2^-48 |c| from the split of c and 2^-22 (|vl| + |cl| + |dl|) from the
 //   two roundings.  The double operations themselves are within 2^-53 (|c|
 //   + 5 D + 8.2 R^2 / (r0 z)) of the real depth (D = the drop; rho^2 within
@@ -209,33 +238,28 @@ __device__ __forceinline__ CapColumn cap_column(const SphereCand &c, float ox)
 __device__ __forceinline__ int cap_fast(const SphereCand &c, const CapColumn &k, float oy, float invf, float invl,
                                         float &d)
 {
-    float sh, sl, dyh, dyl;
-    two_sum(oy, c.dy0h, sh, sl);
-    two_sum(sh, __fadd_rn(sl, c.dy0l), dyh, dyl);
+    float dyh, dyl;
+    offset_pair(oy, c.dy0h, c.dy0l, dyh, dyl);
     const float py = __fmul_rn(dyh, dyh);
     const float pye = __fmaf_rn(dyh, dyh, -py);
-    const float cyt = __fmul_rn(__fmul_rn(2.0f, dyh), dyl);
     float s2, e2, ah, al;
     two_sum(k.s1, -py, s2, e2);
-    two_sum(s2, __fsub_rn(__fsub_rn(__fadd_rn(k.low, e2), pye), cyt), ah, al);
+    two_sum(s2, __fsub_rn(__fadd_rn(k.low, e2), __fmaf_rn(2.0f * dyh, dyl, pye)), ah, al);
     const float my = fabsf(oy) + fabsf(c.dy0h);
     const float ea = 4.547473508864641e-13f * (k.ex + py + my * (my + c.cya));   // 2^-41
-    const float lim = 9.094947017729282e-13f * c.r2h;                     // 2^-40 R^2
-    if (!(ah > 4.0f * ea && ah > lim))
-        return ah < -(4.0f * ea + lim) ? 0 : -1;
-    const float r0 = __fsqrt_rn(ah);
-    const float rr = __fdividef(1.0f, r0);                                 // 1 / r0 within 2 ulp
-    const float corr = __fmul_rn(__fadd_rn(__fmaf_rn(-r0, r0, ah), al), __fmul_rn(0.5f, rr));
+    if (!(ah > 4.0f * ea))
+        return ah < -6.0f * ea ? 0 : -1;
+    const float y = rsqrt_approx(ah);
+    const float r0 = __fmul_rn(ah, y);
+    const float corr = __fmul_rn(__fadd_rn(__fmaf_rn(-r0, r0, ah), al), __fmul_rn(0.5f, y));
     const float dh = __fmul_rn(r0, invf);
     const float dl = __fmaf_rn(r0, invl, __fmaf_rn(corr, invf, __fmaf_rn(r0, invf, -dh)));
     float vh, vl, f, r;
     two_sum(c.ch, -dh, vh, vl);
     two_sum(vh, __fsub_rn(__fadd_rn(vl, c.cl), dl), f, r);               // f + r = the float-float depth
-    const float B = 7.105427357601002e-15f * fabsf(c.ch)                                  // 2^-47
-                    + invf * (9.094947017729282e-13f * r0                                  // 2^-40
-                              + (1.01f * ea + 8.881784197001252e-16f * c.r2h) * rr)       // 2^-50
-                    + 2.384185791015625e-07f * (fabsf(vl) + fabsf(c.cl) + fabsf(dl))       // 2^-22
-                    + 7.52316384526264e-37f;                                               // 2^-120
+    // b0 = 2^-47 |ch| + 2^-22 |cl| + 2^-120; 2^-50 R^2 <= 2^-9 E_A
+    const float B = c.b0 + invf * (9.094947017729282e-13f * r0 + 1.02f * ea * y)          // 2^-40
+                    + 2.384185791015625e-07f * (fabsf(vl) + fabsf(dl));                   // 2^-22
     // half the gap from f to the float on r's side: 2^(e-24) for f in
     // [2^e, 2^(e+1)), 2^(e-25) below a power of two; positive normal f only
     const unsigned bits = __float_as_uint(f), ef = bits >> 23;
@@ -309,11 +333,20 @@ __device__ __forceinline__ void cull_round(const rbsm_occluders &occ, const Floa
         if (keep_r) {
             rc.uxf = f.ux;
             rc.uyf = f.uy;
-            rc.haf = f.ha;
-            rc.hbf = f.hb;
             const float mag = fabsf(dx) + fabsf(dy);
-            rc.es = err_bound(fabsf(rc.s0) + f.ha + spread + mag) + f.ea;
-            rc.et = err_bound(fabsf(rc.t0) + f.hb + spread + mag) + f.ea;
+            const float es = err_bound(fabsf(rc.s0) + f.ha + spread + mag) + f.ea;
+            const float et = err_bound(fabsf(rc.t0) + f.hb + spread + mag) + f.ea;
+            rc.s_out = f.ha + es;
+            rc.s_in = f.ha - es;
+            rc.t_out = f.hb + et;
+            rc.t_in = f.hb - et;
+            // a block's texel centres are within 15.5 along x and 1.5 along y of its centre
+            const float ss = 15.5f * fabsf(f.ux) + 1.5f * fabsf(f.uy) + 2.0f * es;
+            const float st = 15.5f * fabsf(f.uy) + 1.5f * fabsf(f.ux) + 2.0f * et;
+            rc.bs_out = f.ha + ss;
+            rc.bs_in = f.ha - ss;
+            rc.bt_out = f.hb + st;
+            rc.bt_in = f.hb - st;
             rc.depth = f.depth;
             rc.k = k;
             buf[threadIdx.x].r = rc;
@@ -327,11 +360,12 @@ __device__ __forceinline__ void cull_round(const rbsm_occluders &occ, const Floa
         const float rr = f.r + kCullSlack;
         keep_s = gx * gx + gy * gy <= rr * rr;
         if (keep_s) {
-            sc.r2f = f.r * f.r;
+            const float r2f = f.r * f.r;
             const float far = fabsf(sc.dx0) + fabsf(sc.dy0) + 2.0f * h + f.r + f.ea;
-            sc.e = err_bound(far * far) + 2.0f * far * f.ea;
+            const float e2 = err_bound(far * far) + 2.0f * far * f.ea;
+            sc.r_out = r2f + e2;
+            sc.rb_out = r2f + 2.0f * e2;
             sc.dmin = f.dmin;
-            sc.k = k;
             // tile centre - disc centre in float-float: (tc - cx_f) exactly
             // (TwoSum), then the dropped part of the centre
             float a, e;
@@ -342,7 +376,8 @@ __device__ __forceinline__ void cull_round(const rbsm_occluders &occ, const Floa
             sc.r2h = f.r2h; sc.r2l = f.r2l; sc.ch = f.ch; sc.cl = f.cl;
             sc.cxa = fabsf(f.cx);
             sc.cya = fabsf(f.cy);
-            sc.fast = fast && f.fast && sc.cxa <= 1e15f && sc.cya <= 1e15f;
+            sc.b0 = 7.105427357601002e-15f * fabsf(f.ch) + 2.384185791015625e-07f * fabsf(f.cl) + 7.52316384526264e-37f;
+            sc.k = fast && f.fast && sc.cxa <= 1e15f && sc.cya <= 1e15f ? k : ~k;
             buf[threadIdx.x].s = sc;
         }
     }
@@ -438,13 +473,11 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
             const float ox = __fsub_rn(small_int_float(bi + lane), h), oy0 = by - 1.5f;
             for (int q = 0; q < nr; ++q) {
                 const RectCand &r = buf[sm.idx[q]].r;
-                // the block against the rectangle: |s| within 15.5 |ux| + 1.5 |uy| of its centre's
+                // the block against the rectangle
                 const float sb = fabsf(r.s0 + (bx * r.uxf + by * r.uyf)), tb = fabsf(r.t0 + (by * r.uxf - bx * r.uyf));
-                const float ss = 15.5f * fabsf(r.uxf) + 1.5f * fabsf(r.uyf) + 2.0f * r.es;
-                const float st = 15.5f * fabsf(r.uyf) + 1.5f * fabsf(r.uxf) + 2.0f * r.et;
-                if (sb > r.haf + ss || tb > r.hbf + st)
+                if (sb > r.bs_out || tb > r.bt_out)
                     continue;                              // surely outside
-                if (sb + ss < r.haf && tb + st < r.hbf) {
+                if (sb < r.bs_in && tb < r.bt_in) {
 #pragma unroll
                     for (int p = 0; p < kBlockRows; ++p)   // surely covers the block
                         best[p] = r.depth < best[p] ? r.depth : best[p];
@@ -456,9 +489,9 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
                     const float oy = oy0 + (float)p;
                     const float sf = fabsf(r.s0 + (sx + oy * r.uyf));
                     const float tf = fabsf(r.t0 + (tx_ + oy * r.uxf));
-                    if (sf > r.haf + r.es || tf > r.hbf + r.et || !(r.depth < best[p]))
+                    if (sf > r.s_out || tf > r.t_out || !(r.depth < best[p]))
                         continue;                          // surely outside, or it cannot lower the depth
-                    bool in = sf < r.haf - r.es && tf < r.hbf - r.et;
+                    bool in = sf < r.s_in && tf < r.t_in;
                     if (!in)
                         in = rect_covers_exact(occ.rects + r.k, i0 + bi + lane, j0 + bj + p);     // near an edge
                     if (in)
@@ -469,7 +502,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
                 const SphereCand &c = buf[sm.idx[nr + q]].s;
                 // the disc against the block's box of texel centres
                 const float gx = fmaxf(fabsf(c.dx0 + bx) - 15.5f, 0.0f), gy = fmaxf(fabsf(c.dy0 + by) - 1.5f, 0.0f);
-                if (gx * gx + gy * gy > c.r2f + 2.0f * c.e)
+                if (gx * gx + gy * gy > c.rb_out)
                     continue;                              // surely outside
                 const float dxf = c.dx0 + ox;
                 const CapColumn col = cap_column(c, ox);
@@ -480,11 +513,11 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
                 for (int p = 0; p < kBlockRows; ++p) {
                     const float dyf = c.dy0 + oy;
                     // skip when it cannot lower the depth, or surely outside the disc
-                    if (c.dmin < best[0] && !(dxf * dxf + dyf * dyf > c.r2f + c.e)) {
+                    if (c.dmin < best[0] && !(dxf * dxf + dyf * dyf > c.r_out)) {
                         float d = 0.0f;
-                        const int cap = c.fast ? cap_fast(c, col, oy, scale_hi, scale_lo, d) : -1;
+                        const int cap = c.k >= 0 ? cap_fast(c, col, oy, scale_hi, scale_lo, d) : -1;
                         if (cap < 0)
-                            d = cap_depth_exact(occ.spheres + c.k, i0 + bi + lane, j0 + bj + p, inv_zscale, occ.zscale);
+                            d = cap_depth_exact(occ.spheres + (c.k >= 0 ? c.k : ~c.k), i0 + bi + lane, j0 + bj + p, inv_zscale, occ.zscale);
                         if (cap != 0 && d < best[0])
                             best[0] = d;
                     }
