@@ -418,8 +418,9 @@ __device__ __forceinline__ void cull_round(const rbsm_occluders &occ, const Floa
 // the warps turn survivors down (or take a rectangle over the whole of a
 // block) block by block: 8192^2 texels with 140 rectangles and 60 spheres,
 // 4 maps in a call, 202 us a map with tiles of 32 and 150 with 64 (96: 161,
-// 128: 160; blocks handed to the warps one at a time: 163).  One map's 268 MB
-// take 40 us at the copy rate.
+// 128: 160; blocks handed to the warps one at a time: 163); the reciprocal
+// root, the FastTwoSums and the thresholds formed at the cull took the 150 to
+// 143.  One map's 268 MB take 40 us at the copy rate.
 template <bool COPIES, int kTile>
 __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_occluders occ, float *__restrict__ depth,
                                                                 int width, int height, long long pitch,
