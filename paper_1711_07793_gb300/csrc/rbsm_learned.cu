@@ -59,15 +59,17 @@ __global__ void refresh_kernel(void *base)
 }
 
 // One Adam update (Kingma and Ba, Algorithm 1) of parameter p with gradient
-// g; refreshes the BF16 copy.
-__device__ __forceinline__ void adam_update(const State &s, int p, float g, float lr, float bc1, float bc2)
+// g from its moments m0, v0 and value w0 (as they are in the state); refreshes
+// the BF16 copy.
+__device__ __forceinline__ void adam_update(const State &s, int p, float g, float m0, float v0, float w0, float lr,
+                                            float bc1, float bc2)
 {
     constexpr float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float m = b1 * s.m[p] + (1.0f - b1) * g;
-    const float v = b2 * s.v[p] + (1.0f - b2) * g * g;
+    const float m = b1 * m0 + (1.0f - b1) * g;
+    const float v = b2 * v0 + (1.0f - b2) * g * g;
     s.m[p] = m;
     s.v[p] = v;
-    const float val = s.master[p] - lr * (m / bc1) / (sqrtf(v / bc2) + eps);
+    const float val = w0 - lr * (m / bc1) / (sqrtf(v / bc2) + eps);
     s.master[p] = val;
     write_copies(s, p, val);
 }
@@ -79,7 +81,7 @@ __global__ void adam_kernel(void *base, float lr, float bc1, float bc2)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const State s = state_of(base);
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < kParams; p += gridDim.x * blockDim.x) {
-        adam_update(s, p, s.grad[p], lr, bc1, bc2);
+        adam_update(s, p, s.grad[p], s.m[p], s.v[p], s.master[p], lr, bc1, bc2);
         s.grad[p] = 0.0f;
     }
 }
@@ -135,8 +137,10 @@ __global__ void dataset_kernel(const MapDev m, const float *__restrict__ x, cons
 // ----------------------------------------------------------- training --
 //
 // Gradient and forward pass on the fifth-generation tensor cores.  A CTA of
-// 128 threads takes tiles of 128 samples (M = 128, one TMEM lane and one
-// thread per sample).  Per tile, with one thread issuing every product:
+// 256 threads takes tiles of 128 samples (M = 128, one TMEM lane per sample;
+// a sample's row is shared by two threads, 32 of its 64 units each: warps w
+// and w + 4 read the same lanes).  Per tile, with one thread issuing every
+// product:
 //
 //   forward        a1 = X W1,  a2 = h1 W2,  y = h2 W3             (K-major A and B)
 //   backward-data  dh2 = dY W3^T,  dh1 = dA2 W2^T                  (B: the forward
@@ -152,15 +156,23 @@ __global__ void dataset_kernel(const MapDev m, const float *__restrict__ x, cons
 // descriptor over the same bytes is that activation transposed (units
 // along M or N, samples along K) for the weight-gradient products, which
 // accumulate in TMEM across the CTA's tiles.  The epilogues (bias, ReLU
-// and its mask, loss, BF16 rounding) are per thread on its own row.
+// and its mask, loss, BF16 rounding) are per thread on its own half row.
+//
+// Bound: the chain of six dependent products and epilogues of a tile (the
+// tensor pipe is 5 % active).  Against one thread per sample, the output
+// layer's weight gradient ahead of the commit and a reduction that read what
+// Adam needs after its sums, a step (gradient + Adam) of 20000 samples went
+// from 16.8 to 14.9 us, of 65536 from 25.8 to 22.8, and of 8192 from 12.0 to
+// the 11 us that its two launches take on the host.  The same bits.
 //
 // Bias gradients and the loss are FP32 column sums of unrounded values in a
-// fixed order (a butterfly over the warp, then the four warps in order).
+// fixed order (a butterfly over the warp, then the four row groups in order).
 // Each CTA writes its sums to its row of the partials; the reduction kernel
 // adds the rows in CTA order, so a gradient is bit-reproducible.
 
 constexpr int kTcRows = 128;                       // samples per tile (M)
-constexpr int kTcThreads = 128;
+constexpr int kTcThreads = 2 * kTcRows;            // two threads per sample
+constexpr int kHalf = kHid / 2;                    // hidden units per thread
 constexpr int kActCols = kIn + 2 * kHid;           // X | H1 | H2
 constexpr int kGrdCols = 2 * kHid + 16;            // dA1 | dA2 | dY (padded to 16)
 constexpr uint32_t kCore = 128;                    // bytes per core matrix = LBO of a K-major buffer
@@ -210,12 +222,13 @@ __device__ __forceinline__ void stage_weights(unsigned char *dst, const uint16_t
     }
 }
 
-// Column sums of v[0..64) over the warp's 32 lanes by halving exchanges:
-// lane L returns the sums of columns 2L and 2L + 1.  v is consumed.
-__device__ __forceinline__ float2 warp_column_sums(float (&v)[kHid], unsigned lane)
+// Column sums of v[0..32) over the warp's 32 lanes by halving exchanges:
+// lane L returns the sum of column L.  v is consumed.
+__device__ __forceinline__ float warp_column_sums(float (&v)[kHalf], unsigned lane)
 {
+    static_assert(kHalf == 32, "one column per lane");
 #pragma unroll
-    for (int width = 32, bit = 16; bit >= 1; width >>= 1, bit >>= 1) {
+    for (int width = 16, bit = 16; bit >= 1; width >>= 1, bit >>= 1) {
         const bool upper = (lane & bit) != 0;
 #pragma unroll
         for (int i = 0; i < width; ++i) {
@@ -224,7 +237,7 @@ __device__ __forceinline__ float2 warp_column_sums(float (&v)[kHid], unsigned la
             v[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
         }
     }
-    return make_float2(v[0], v[1]);
+    return v[0];
 }
 
 __device__ __forceinline__ float warp_sum(float v)
@@ -258,22 +271,22 @@ __device__ __forceinline__ bool wait_products(uint64_t *bar, uint32_t &parity)
     return all;
 }
 
-// Bias, ReLU and BF16 rounding of one hidden layer's row (FP32 accumulators
-// a[64]); writes h into eight column groups of act and returns the ReLU mask
-// (bit j: unit j positive).
-__device__ __forceinline__ uint64_t hidden_epilogue(const float (&a)[kHid], const float *bias, unsigned char *act,
+// Bias, ReLU and BF16 rounding of half a hidden layer's row (FP32
+// accumulators a[32], biases from bias[0]); writes h into four column groups
+// of act and returns the ReLU mask (bit j: unit j positive).
+__device__ __forceinline__ uint32_t hidden_epilogue(const float (&a)[kHalf], const float *bias, unsigned char *act,
                                                     int row, int group0)
 {
-    uint64_t mask = 0;
+    uint32_t mask = 0;
 #pragma unroll
-    for (int g = 0; g < kHid / 8; ++g) {
+    for (int g = 0; g < kHalf / 8; ++g) {
         uint32_t w[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int j = g * 8 + 2 * q;
             const float v0 = a[j] + bias[j], v1 = a[j + 1] + bias[j + 1];
-            mask |= (uint64_t)(v0 > 0.0f) << j;
-            mask |= (uint64_t)(v1 > 0.0f) << (j + 1);
+            mask |= (uint32_t)(v0 > 0.0f) << j;
+            mask |= (uint32_t)(v1 > 0.0f) << (j + 1);
             w[q] = pack_bf16(fmaxf(v0, 0.0f), fmaxf(v1, 0.0f));
         }
         *reinterpret_cast<uint4 *>(group_ptr(act, kActSbo, row, group0 + g)) = make_uint4(w[0], w[1], w[2], w[3]);
@@ -281,24 +294,22 @@ __device__ __forceinline__ uint64_t hidden_epilogue(const float (&a)[kHid], cons
     return mask;
 }
 
-// Mask a backward row by the ReLU mask, write it (BF16) into eight column
-// groups of grd, and leave this warp's FP32 column sums in red[warp].
-__device__ __forceinline__ void backward_epilogue(float (&d)[kHid], uint64_t mask, unsigned char *grd, int row,
-                                                  int group0, float (*red)[kHid], int warp, unsigned lane)
+// Mask half a backward row by the ReLU mask, write it (BF16) into four column
+// groups of grd, and leave this warp's FP32 column sums in red[0..32).
+__device__ __forceinline__ void backward_epilogue(float (&d)[kHalf], uint32_t mask, unsigned char *grd, int row,
+                                                  int group0, float *red, unsigned lane)
 {
 #pragma unroll
-    for (int j = 0; j < kHid; ++j)
+    for (int j = 0; j < kHalf; ++j)
         d[j] = ((mask >> j) & 1u) ? d[j] : 0.0f;
 #pragma unroll
-    for (int g = 0; g < kHid / 8; ++g) {
+    for (int g = 0; g < kHalf / 8; ++g) {
         const int j = g * 8;
         *reinterpret_cast<uint4 *>(group_ptr(grd, kGrdSbo, row, group0 + g)) =
             make_uint4(pack_bf16(d[j], d[j + 1]), pack_bf16(d[j + 2], d[j + 3]), pack_bf16(d[j + 4], d[j + 5]),
                        pack_bf16(d[j + 6], d[j + 7]));
     }
-    const float2 s = warp_column_sums(d, lane);
-    red[warp][2 * lane] = s.x;
-    red[warp][2 * lane + 1] = s.y;
+    red[lane] = warp_column_sums(d, lane);
 }
 
 // kTrain: gradient of the mean loss over samples[order[0..n)] into the
@@ -306,7 +317,7 @@ __device__ __forceinline__ void backward_epilogue(float (&d)[kHid], uint64_t mas
 // of samples[0..n).  Launched as a programmatic dependent (it waits for the
 // previous kernel before reading global memory).
 template <bool kTrain>
-__global__ void __launch_bounds__(kTcThreads)
+__global__ void __launch_bounds__(kTcThreads, 2)
 surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int *__restrict__ order, long long n,
                     float inv_batch, float *__restrict__ out)
 {
@@ -314,12 +325,16 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
     TcSmem &sm = *reinterpret_cast<TcSmem *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5;
     const unsigned lane = lane_id();
+    // the thread's sample of a tile (also its TMEM lane) and half of the
+    // hidden units; quarter: the warp's group of 32 samples
+    const int row = tid & (kTcRows - 1), half = tid / kTcRows, quarter = warp & 3;
 
     if (tid == 0)
         tc::mbar_init(&sm.bar, 1);
     if (warp == 0)
         tc::tmem_alloc(&sm.tmem_base, kTmemCols);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    sync_for_mma(false);                       // the barrier and the TMEM address
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     const State st = state_of(base);
@@ -328,7 +343,7 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
     // weights are staged), so the gather overlaps the previous tile's products
     auto gather = [&](long long tile) {
         rbsm_sample v{0u, 0.0f, 0.0f, 0.0f, 0.0f};
-        const long long b = tile * kTcRows + tid;
+        const long long b = tile * kTcRows + row;
         if (tile < tiles && b < n)
             v = data[kTrain ? (long long)order[b] : b];
         return v;
@@ -343,12 +358,14 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
     }
     if (tid < kOut)
         sm.b3[tid] = st.master[kOffB3 + tid];
-    if (kTrain)   // dY columns 8..15 stay zero
-        *reinterpret_cast<uint4 *>(group_ptr(sm.grd, kGrdSbo, tid, kGdY + 1)) = make_uint4(0u, 0u, 0u, 0u);
-    bool fail = sync_for_mma(false);
+    if (kTrain && half == 1)   // dY columns 8..15 stay zero
+        *reinterpret_cast<uint4 *>(group_ptr(sm.grd, kGrdSbo, row, kGdY + 1)) = make_uint4(0u, 0u, 0u, 0u);
+    // (the first tile's barrier below hands the weights over as well)
+    bool fail = false;
 
     const uint32_t tmem = sm.tmem_base;
-    const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
+    const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
+    const uint32_t half_off = lane_off + (uint32_t)(half * kHalf);       // this thread's half row
     const uint32_t tA = tmem + kColA, tB = tmem + kColB, tP1 = tmem + kColP1, tP2 = tmem + kColP2;
     const uint32_t act = tc::smem_addr(sm.act), grd = tc::smem_addr(sm.grd);
     const uint32_t w1t = tc::smem_addr(sm.w1t), w2t = tc::smem_addr(sm.w2t), w3t = tc::smem_addr(sm.w3t);
@@ -362,7 +379,7 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
     bool first = true, p1_pending = false;
     float db1 = 0.0f, db2 = 0.0f, db3 = 0.0f, loss = 0.0f;    // thread t: column t of b1 / b2 (t < 64), b3 (t < 2)
     for (long long tile = blockIdx.x; tile < tiles && !fail; tile += gridDim.x) {
-        const long long b = tile * kTcRows + tid;
+        const long long b = tile * kTcRows + row;
         const bool valid = b < n;
         if (p1_pending) {       // the previous tile's weight-gradient products still read act and grd
             const bool ok = wait_products(&sm.bar, parity);
@@ -371,7 +388,7 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
             if ((fail = sync_for_mma(!ok)))
                 break;
         }
-        {   // input row: 25 pattern bits, fx, fy, gap, zeros (BF16)
+        {   // input row: 25 pattern bits, fx, fy, gap, zeros (BF16); 16 columns per thread
             uint32_t w[16];
 #pragma unroll
             for (int k = 0; k < 12; ++k) {
@@ -383,9 +400,10 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
             w[14] = 0u;
             w[15] = 0u;
 #pragma unroll
-            for (int g = 0; g < 4; ++g)
-                *reinterpret_cast<uint4 *>(group_ptr(sm.act, kActSbo, tid, kGX + g)) =
-                    make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3]);
+            for (int g = 0; g < 2; ++g)
+                *reinterpret_cast<uint4 *>(group_ptr(sm.act, kActSbo, row, kGX + 2 * half + g)) =
+                    half == 0 ? make_uint4(w[4 * g], w[4 * g + 1], w[4 * g + 2], w[4 * g + 3])
+                              : make_uint4(w[8 + 4 * g], w[9 + 4 * g], w[10 + 4 * g], w[11 + 4 * g]);
         }
         const float label = smp.label;
         smp = gather(tile + gridDim.x);
@@ -400,11 +418,11 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
             tc::commit(&sm.bar);
         }
         bool ok = wait_products(&sm.bar, parity);
-        uint64_t mask1 = 0, mask2 = 0;
+        uint32_t mask1 = 0, mask2 = 0;
         if (ok) {
-            float a[kHid];
-            tc::tmem_load_row<kHid>(tA + lane_off, a);
-            mask1 = hidden_epilogue(a, sm.b1, sm.act, tid, kGH1);
+            float a[kHalf];
+            tc::tmem_load_row<kHalf>(tA + half_off, a);
+            mask1 = hidden_epilogue(a, sm.b1 + half * kHalf, sm.act, row, kGH1 + half * (kHalf / 8));
         }
         if ((fail = sync_for_mma(!ok)))
             break;
@@ -418,9 +436,9 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
         }
         ok = wait_products(&sm.bar, parity);
         if (ok) {
-            float a[kHid];
-            tc::tmem_load_row<kHid>(tB + lane_off, a);
-            mask2 = hidden_epilogue(a, sm.b2, sm.act, tid, kGH2);
+            float a[kHalf];
+            tc::tmem_load_row<kHalf>(tB + half_off, a);
+            mask2 = hidden_epilogue(a, sm.b2 + half * kHalf, sm.act, row, kGH2 + half * (kHalf / 8));
         }
         if ((fail = sync_for_mma(!ok)))
             break;
@@ -433,7 +451,7 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
             tc::commit(&sm.bar);
         }
         ok = wait_products(&sm.bar, parity);
-        if (ok) {
+        if (ok && half == 0) {
             uint32_t r[2];
             tc::tmem_ld2(tA + lane_off, r);
             const float y0 = __uint_as_float(r[0]) + sm.b3[0], y1 = __uint_as_float(r[1]) + sm.b3[1];
@@ -454,7 +472,7 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
                     dy1 = 2.0f * re * inv_batch;
                     l = __fadd_rn(__fmul_rn(rv, rv), __fmul_rn(re, re));
                 }
-                *reinterpret_cast<uint4 *>(group_ptr(sm.grd, kGrdSbo, tid, kGdY)) =
+                *reinterpret_cast<uint4 *>(group_ptr(sm.grd, kGrdSbo, row, kGdY)) =
                     make_uint4(pack_bf16(dy0, dy1), 0u, 0u, 0u);
                 const float s0 = warp_sum(dy0), s1 = warp_sum(dy1), sl = warp_sum(l);
                 if (lane == 0) {
@@ -475,22 +493,23 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
             db3 += ((sm.red3[0][tid] + sm.red3[1][tid]) + sm.red3[2][tid]) + sm.red3[3][tid];
         if (tid == 0)
             loss += ((sm.red3[0][2] + sm.red3[1][2]) + sm.red3[2][2]) + sm.red3[3][2];
-        // ---- dh2 = dY W3^T (K = 16) and dW3 += [H1 | H2]^T dY (K = the tile's 128 samples)
+        // ---- dh2 = dY W3^T (K = 16), then, under its epilogue, dW3 += [H1 | H2]^T dY (K = the
+        // tile's 128 samples; the next commit covers them)
         if (tid == 0) {
             tc::mma_bf16(tB, tc::smem_desc(grd + kGdY * kCore, kCore, kGrdSbo),
                          tc::smem_desc(w3t, kW3tSbo, kCore), id64_bmn, false);
+            tc::commit(&sm.bar);
 #pragma unroll
             for (int k = 0; k < kTcRows / 16; ++k)
                 tc::mma_bf16(tP2, tc::smem_desc(act + kGH1 * kCore + k * 2 * kActSbo, kActSbo, kCore),
                              tc::smem_desc(grd + kGdY * kCore + k * 2 * kGrdSbo, kGrdSbo, kCore), idP2,
                              !(first && k == 0));
-            tc::commit(&sm.bar);
         }
         ok = wait_products(&sm.bar, parity);
         if (ok) {
-            float d[kHid];
-            tc::tmem_load_row<kHid>(tB + lane_off, d);
-            backward_epilogue(d, mask2, sm.grd, tid, kGdA2, sm.red2, warp, lane);
+            float d[kHalf];
+            tc::tmem_load_row<kHalf>(tB + half_off, d);
+            backward_epilogue(d, mask2, sm.grd, row, kGdA2 + half * (kHalf / 8), sm.red2[quarter] + half * kHalf, lane);
         }
         if ((fail = sync_for_mma(!ok)))
             break;
@@ -506,9 +525,9 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
             db2 += ((sm.red2[0][tid] + sm.red2[1][tid]) + sm.red2[2][tid]) + sm.red2[3][tid];
         ok = wait_products(&sm.bar, parity);
         if (ok) {
-            float d[kHid];
-            tc::tmem_load_row<kHid>(tA + lane_off, d);
-            backward_epilogue(d, mask1, sm.grd, tid, kGdA1, sm.red1, warp, lane);
+            float d[kHalf];
+            tc::tmem_load_row<kHalf>(tA + half_off, d);
+            backward_epilogue(d, mask1, sm.grd, row, kGdA1 + half * (kHalf / 8), sm.red1[quarter] + half * kHalf, lane);
         }
         if ((fail = sync_for_mma(!ok)))
             break;
@@ -533,25 +552,25 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
         if (ok) {
             // row r of the weight-gradient accumulators: r < 64 is unit r of dA1
             // (columns 0..31: dW1[i][r]); r >= 64 is unit r - 64 of dA2 (columns
-            // 32..95: dW2[i][r - 64]) and of H2 in the dW3 product
+            // 32..95: dW2[i][r - 64], 32 per thread) and of H2 in the dW3 product
             float *part = st.part + (size_t)blockIdx.x * kPartStride;
-            float d[kIn + kHid];
-            tc::tmem_load_row<kIn + kHid>(tP1 + lane_off, d);
-            uint32_t r3[2];
-            tc::tmem_ld2(tP2 + lane_off, r3);
-            if (tid < kHid) {
+            if (row >= kHid || half == 0) {       // uniform over a warp
+                float d[kHalf];
+                tc::tmem_load_row<kHalf>(tP1 + lane_off + (row < kHid ? 0u : (uint32_t)(kIn + half * kHalf)), d);
+                float *dst = row < kHid ? part + kOffW1 + row : part + kOffW2 + half * kHalf * kHid + (row - kHid);
 #pragma unroll
-                for (int i = 0; i < kIn; ++i)
-                    part[kOffW1 + i * kHid + tid] = d[i];
+                for (int i = 0; i < kHalf; ++i)
+                    dst[i * kHid] = d[i];
+            }
+            if (row >= kHid && half == 1) {
+                uint32_t r3[2];
+                tc::tmem_ld2(tP2 + lane_off, r3);
+                part[kOffW3 + (row - kHid) * kOut] = __uint_as_float(r3[0]);
+                part[kOffW3 + (row - kHid) * kOut + 1] = __uint_as_float(r3[1]);
+            }
+            if (tid < kHid) {
                 part[kOffB1 + tid] = db1;
                 part[kOffB2 + tid] = db2;
-            } else {
-                const int o = tid - kHid;
-#pragma unroll
-                for (int i = 0; i < kHid; ++i)
-                    part[kOffW2 + i * kHid + o] = d[kIn + i];
-                part[kOffW3 + o * kOut] = __uint_as_float(r3[0]);
-                part[kOffW3 + o * kOut + 1] = __uint_as_float(r3[1]);
             }
             if (tid < kOut)
                 part[kOffB3 + tid] = db3;
@@ -570,32 +589,49 @@ surrogate_tc_kernel(void *base, const rbsm_sample *__restrict__ data, const int 
 }
 
 // Sum of the `parts` partial rows of every parameter (and the loss), in CTA
-// order within each of 8 strided subsets, the 8 subset sums then combined
-// by a fixed butterfly.  step = 0: added to the gradient.  step > 0: one Adam
-// step with (gradient + sum), and the gradient cleared.
+// order within each of 8 strided subsets (one per warp, a lane per
+// parameter), the 8 subset sums then combined in a fixed tree.  step = 0:
+// added to the gradient.  step > 0: one Adam step with (gradient + sum), and
+// the gradient cleared.  What the update reads is loaded before the sums.
 constexpr int kReduceLanes = 8;
-__global__ void __launch_bounds__(256) reduce_kernel(void *base, int parts, int step, float lr, float bc1, float bc2)
+__global__ void __launch_bounds__(32 * kReduceLanes) reduce_kernel(void *base, int parts, int step, float lr,
+                                                                   float bc1, float bc2)
 {
+    // no launch_dependents here: the next gradient kernel's CTAs, early on the
+    // SMs, took a step of 32768 samples from 15.2 to 18.7 us
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    __shared__ float sub[kReduceLanes][32];
     const State s = state_of(base);
-    const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int p = gtid / kReduceLanes, q = gtid % kReduceLanes;
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const int p = blockIdx.x * 32 + lane;
+    float g = 0.0f, m = 0.0f, v = 0.0f, w = 0.0f;
+    if (q == 0 && p < kParams) {
+        g = s.grad[p];
+        if (step > 0) {
+            m = s.m[p];
+            v = s.v[p];
+            w = s.master[p];
+        }
+    }
     float sum = 0.0f;
-    if (p <= kParams)
+    if (p <= kParams) {
+#pragma unroll 8
         for (int c = q; c < parts; c += kReduceLanes)
             sum += s.part[(size_t)c * kPartStride + p];
-#pragma unroll
-    for (int bit = kReduceLanes / 2; bit >= 1; bit >>= 1)
-        sum += __shfl_xor_sync(0xffffffffu, sum, bit);
+    }
+    sub[q][lane] = sum;
+    __syncthreads();
     if (q != 0 || p > kParams)
         return;
+    sum = ((sub[0][lane] + sub[4][lane]) + (sub[2][lane] + sub[6][lane])) +
+          ((sub[1][lane] + sub[5][lane]) + (sub[3][lane] + sub[7][lane]));
     if (p == kParams) {
         s.loss[0] += sum;
         return;
     }
-    const float g = s.grad[p] + sum;
+    g += sum;
     if (step > 0) {
-        adam_update(s, p, g, lr, bc1, bc2);
+        adam_update(s, p, g, m, v, w, lr, bc1, bc2);
         s.grad[p] = 0.0f;
     } else {
         s.grad[p] = g;
@@ -650,8 +686,8 @@ int launch_reduce(void *state, int parts, int step, float lr, cudaStream_t strea
         bc1 = 1.0 - pow(0.9, (double)step);
         bc2 = 1.0 - pow(0.999, (double)step);
     }
-    const int threads = 256;
-    const int blocks = ((kParams + 1) * kReduceLanes + threads - 1) / threads;
+    const int threads = 32 * kReduceLanes;
+    const int blocks = (kParams + 1 + 31) / 32;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.blockDim = dim3(threads);
