@@ -16,6 +16,14 @@ int check_frags(const rbsm_frags *f);
 int check_params(const rbsm_params *p, int *max_dist);
 // True when [out, out + bytes) overlaps the fragment planes or the map.
 bool overlaps_inputs(const rbsm_map &m, const rbsm_frags &f, const void *out, size_t bytes);
+
+// rbsm_visibility (mode RBSM_MODE_SILHOUETTE) and rsmss_filter
+// (RBSM_MODE_FILTER): argument checks and launch.  plain_large: whether n
+// fragments have tiles enough for its CTAs of 1024 threads.
+int plain_entry(int mode, const rbsm_map *map, const rbsm_frags *frags, float *vis, uint16_t *codes,
+                const rbsm_params *params, void *stream);
+bool plain_large(int64_t n, int sms);
+
 bool aligned16(const void *p);
 int device_sm_count();
 MapDev to_dev(const rbsm_map &m);

@@ -164,6 +164,8 @@ plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restric
 // 1024, 53.1 / 23.0 with two of 640, 52.2 / 24.4 with four of 320, 54.3 / 23.3
 // with five of 256 (before the walks' pairs of steps and the runs of 16:
 // 49.2 / 20.2 now).
+bool plain_large(int64_t n, int sms) { return (n + kWarpTile - 1) / kWarpTile >= 32LL * sms; }
+
 template <int MODE, bool CODES, int kThreads>
 int launch_plain(const rbsm_map &map, const rbsm_frags &f, float *sil, float *fil, uint16_t *codes,
                  int max_dist, int sms, cudaStream_t stream)
@@ -198,8 +200,7 @@ int launch_plain(const rbsm_map &map, const rbsm_frags &f, float *sil, float *fi
     const int sms = device_sm_count();
     if (sms <= 0)
         return cuda_fail(cudaErrorNoDevice);
-    const long long warp_tiles = (f.n + kWarpTile - 1) / kWarpTile;
-    return warp_tiles >= 32LL * sms
+    return plain_large(f.n, sms)
                ? launch_plain<MODE, CODES, 1024>(map, f, sil, fil, codes, max_dist, sms, stream)
                : launch_plain<MODE, CODES, 256>(map, f, sil, fil, codes, max_dist, sms, stream);
 }

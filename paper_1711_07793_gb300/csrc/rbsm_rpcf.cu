@@ -18,7 +18,7 @@
 // edge samples writes its mean at once, and one outside the shared block
 // (below) walks its own samples, so no second pass is needed.  For k = 1
 // there is nothing to add and the answers are stored as floats
-// (rsmss_filter's bits).  Because the answers do not depend on the order of
+// (rsmss_filter's bits, and its kernel on large textured calls).  Because the answers do not depend on the order of
 // the work, the warps of a CTA share its strips as they come free.
 #include <cuda_runtime.h>
 
@@ -245,7 +245,7 @@ __device__ __forceinline__ void block_bits(const MapDev &m, float u, float v, fl
 // (up to 1152 samples, 36 rounds, at k = 3), and the tiles came from a fixed
 // partition or one at a time from a global counter; 3840x2160 fragments on
 // an 8192^2 map, k = 1 / 3 / 5: 66 / 179 / 488 us with tiles from the
-// counter, 56.7 / 134.5 / 291 us now.
+// counter, 56.8 / 128.7 / 288 us now.
 constexpr unsigned kRun = 8;       // 16: 161.7 against 159.7 us, and 48 against 32.4 us for 320x240 fragments
 
 template <int K, int kThreads>
@@ -518,6 +518,13 @@ int rpcf_entry(const rbsm_map *map, const rbsm_frags *frags, float *vis, int32_t
                 reinterpret_cast<uintptr_t>(vis) < reinterpret_cast<uintptr_t>(ws) + 8u)))
         return RBSM_ERR_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    // k = 1 is rsmss_filter: with a texture and enough tiles for CTAs of 1024
+    // its kernel (3840x2160 / 1277x719 fragments 47.0 / 14.9 against 57.6 /
+    // 16.5 us here); without one, or on few fragments, one strip per warp
+    // finishes sooner (3840x2160 without a texture 76.1 against 80.2 us, one
+    // call on 320x240 22.3 against 25.7)
+    if (k == 1 && map->texture && plain_large(frags->n, device_sm_count()))
+        return plain_entry(RBSM_MODE_FILTER, map, frags, vis, nullptr, params, stream);
     switch (k) {
     case 1: return launch_rpcf<1>(*map, *frags, vis, max_dist, s);
     case 3: return launch_rpcf<3>(*map, *frags, vis, max_dist, s);
