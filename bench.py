@@ -624,7 +624,7 @@ def measure_rpcf(api, maps, xyz, frames, n_frag, args, stream, k=3):
     as RSMSS: the k x k samples re-read texels that are already on chip)."""
     import torch
     outs = [torch.empty(n_frag, dtype=torch.float32, device=xyz[0].device) for _ in range(frames)]
-    ws = torch.zeros(2, dtype=torch.int64, device=xyz[0].device)     # the tile counter of rbsm_rpcf_ws
+    ws = torch.zeros(2, dtype=torch.int64, device=xyz[0].device)     # the workspace rbsm_rpcf_ws takes
     steps = max(3, min(args.steps // 20, 20))
 
     def timed(fn):
