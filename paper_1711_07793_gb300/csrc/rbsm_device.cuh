@@ -498,12 +498,11 @@ struct JobOut {
     int mode;
 };
 
-// Fragment of a warp tile that a lane's element e is: two pairs in vector
-// tiles (8-byte accesses), l, l+32, l+64, l+96 in others (coalesced 4-byte
-// ones).
-__device__ __forceinline__ int tile_slot(bool vec, unsigned lane, int e)
+// Fragment of a warp tile that a lane's element e is: two pairs (8-byte
+// accesses) or l, l+32, l+64, l+96 (coalesced 4-byte ones).
+__device__ __forceinline__ int tile_slot(bool pairs, unsigned lane, int e)
 {
-    return vec ? (e >> 1) * 64 + 2 * (int)lane + (e & 1) : (int)lane + 32 * e;
+    return pairs ? (e >> 1) * 64 + 2 * (int)lane + (e & 1) : (int)lane + 32 * e;
 }
 
 // The coordinates of a tile that is not a vector tile, read directly.
@@ -548,6 +547,11 @@ __device__ __forceinline__ void stage_tile(const WarpTileIO &t, unsigned lane, f
 // single ones 32 apart.)  The buffer is read by other lanes than the one
 // that copied it: a warp barrier after the wait, and another before it is
 // refilled.
+//
+// SINGLES: single fragments 32 apart, for kernels that read a map without a
+// texture: each of a fragment's five loads then covers 32 fragments in a row
+// and touches half the lines.
+template <bool SINGLES = false>
 __device__ __forceinline__ void fetch_tile(const WarpTileIO &t, unsigned lane, const float4 (&buf)[3][32],
                                            LaneCoords &c)
 {
@@ -555,7 +559,13 @@ __device__ __forceinline__ void fetch_tile(const WarpTileIO &t, unsigned lane, c
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncwarp();
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int e = 0; SINGLES && e < kPerThread; ++e) {
+            c.x[e] = reinterpret_cast<const float *>(buf[0])[lane + 32 * e];
+            c.y[e] = reinterpret_cast<const float *>(buf[1])[lane + 32 * e];
+            c.z[e] = reinterpret_cast<const float *>(buf[2])[lane + 32 * e];
+        }
+#pragma unroll
+        for (int h = 0; !SINGLES && h < 2; ++h) {
             const float2 vx = reinterpret_cast<const float2 *>(buf[0])[lane + 32 * h];
             const float2 vy = reinterpret_cast<const float2 *>(buf[1])[lane + 32 * h];
             const float2 vz = reinterpret_cast<const float2 *>(buf[2])[lane + 32 * h];
@@ -614,19 +624,26 @@ __device__ __forceinline__ void drain_queue(const Jobs &jobs, WarpQueue &wq, int
 }
 
 // Classify one warp tile whose coordinates the lane holds, store its answers
-// (provisional for edge fragments) and queue its edge fragments.
-template <int MODE, bool CODES>
+// (provisional for edge fragments) and queue its edge fragments.  TEX: whether
+// the map has a texture, 1 or 0, or -1 to ask the map per tile.  Kernels
+// made for one of them hold half the code, and without a texture (0) a
+// lane's fragments are single ones 32 apart (see fetch_tile; -1 keeps the
+// pairs).  3840x2160 fragments without a texture: filtering 75.2 us with pairs
+// and a kernel for both, 56.4 with TEX 0; silhouette 67.4 and 53.0; depth
+// buffers, 4 frames, 313 and 266 (with a texture 195.4 and 193.4, TEX 1).
+template <int MODE, bool CODES, int TEX = -1>
 __device__ __forceinline__ void classify_warp_tile(const MapDev &m, const WarpTileIO &t, const LaneCoords &c,
                                                    WarpQueue &wq, int &count)
 {
     const unsigned lane = lane_id();
     const unsigned below = (1u << lane) - 1u;
+    const bool pairs = TEX != 0 && t.vec;
     FragResult r[kPerThread];
     uint32_t bits[kPerThread];
     bool edge[kPerThread];
     // classify the lane's four fragments first (no warp-wide step in between,
     // so all their texel loads are issued back to back) ...
-    if (m.tex) {
+    if (TEX < 0 ? m.tex != 0 : TEX != 0) {
         // one branch for the four fragments' eight gathers: tested per
         // fragment, the texture handle put a branch between one fragment's
         // gathers and the next one's (depth buffers, 4 frames of 3840x2160
@@ -650,6 +667,38 @@ __device__ __forceinline__ void classify_warp_tile(const MapDev &m, const WarpTi
             for (int e = 0; e < kPerThread; ++e)
                 edge[e] = edge[e] && tile_slot(false, lane, e) < t.count;
         }
+    } else if (TEX == 0) {
+        // the four fragments' own texels first, then their neighbours, so
+        // that no fragment's loads wait for another's (in silhouette recovery
+        // too, where a shadowed fragment needs none: 1920x1080 20.8 us,
+        // 3840x2160 53.0; branched past when shadowed 21.3 and 53.0, and one
+        // fragment after the other 22.3 and 59.2).  A partial tile's lanes
+        // past its end hold zeros and are masked after.
+        const float *p[kPerThread];
+        float zc[kPerThread];
+        int i[kPerThread], j[kPerThread];
+#pragma unroll
+        for (int e = 0; e < kPerThread; ++e) {
+            float f;
+            texel_of(__fmul_rn(c.x[e], (float)m.width), m.width, i[e], f);
+            texel_of(__fmul_rn(c.y[e], (float)m.height), m.height, j[e], f);
+            p[e] = m.depth + (long long)j[e] * m.pitch + i[e];
+            zc[e] = __ldg(p[e]);
+        }
+        float4 nb[kPerThread];
+#pragma unroll
+        for (int e = 0; e < kPerThread; ++e) {
+            nb[e].x = __ldg(p[e] - (i[e] > 0 ? 1 : 0));
+            nb[e].y = __ldg(p[e] + (i[e] < m.width - 1 ? 1 : 0));
+            nb[e].z = __ldg(p[e] + (j[e] < m.height - 1 ? m.pitch : 0));
+            nb[e].w = __ldg(p[e] - (j[e] > 0 ? m.pitch : 0));
+        }
+#pragma unroll
+        for (int e = 0; e < kPerThread; ++e) {
+            edge[e] = classify_from<MODE, CODES>(c.z[e], zc[e], nb[e].x, nb[e].y, nb[e].z, nb[e].w, r[e], bits[e]);
+            if (!t.vec)
+                edge[e] = edge[e] && tile_slot(false, lane, e) < t.count;
+        }
     } else if (t.vec) {
 #pragma unroll
         for (int e = 0; e < kPerThread; ++e)
@@ -667,7 +716,7 @@ __device__ __forceinline__ void classify_warp_tile(const MapDev &m, const WarpTi
     // ... then queue the edge fragments, one ballot per element
 #pragma unroll
     for (int e = 0; e < kPerThread; ++e) {
-        const int s = tile_slot(t.vec, lane, e);
+        const int s = tile_slot(pairs, lane, e);
         const unsigned mask = __ballot_sync(0xffffffffu, edge[e]);
         if (edge[e]) {
             wq.q[count + __popc(mask & below)] =
@@ -675,7 +724,7 @@ __device__ __forceinline__ void classify_warp_tile(const MapDev &m, const WarpTi
         }
         count += __popc(mask);
     }
-    if (t.vec) {
+    if (pairs) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const long long g = t.first + tile_slot(true, lane, 2 * h);

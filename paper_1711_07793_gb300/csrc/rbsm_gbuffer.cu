@@ -59,7 +59,7 @@ __device__ __forceinline__ void pixel_of(const GBufDev &g, long long f, int &px,
 // planes are kernel parameters, so the hot loop takes them from the
 // constant bank instead of holding them in registers (a launch over many
 // jobs, indexing a job table at run time, measured 35 % slower).
-template <int MODE, bool CODES, int kThreads>
+template <int MODE, bool CODES, int kThreads, int TEX>
 __global__ void __launch_bounds__(kThreads, 1280 / kThreads)
 gbuffer_kernel(const MapDev m, const GBufDev g, float *__restrict__ sil, float *__restrict__ fil,
                uint16_t *__restrict__ codes, int max_dist, bool vec_planes)
@@ -98,13 +98,17 @@ gbuffer_kernel(const MapDev m, const GBufDev g, float *__restrict__ sil, float *
     };
     // the depths of a tile (vector path: contiguous rows)
     auto load = [&](const WarpTileIO &t, float (&d)[kPerThread]) {
-        if (t.vec) {
+        if (TEX != 0 && t.vec) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const float2 v = __ldcs(reinterpret_cast<const float2 *>(g.d + t.first + tile_slot(true, lane, 2 * h)));
                 d[2 * h] = v.x;
                 d[2 * h + 1] = v.y;
             }
+        } else if (t.vec) {
+#pragma unroll
+            for (int e = 0; e < kPerThread; ++e)
+                d[e] = __ldcs(g.d + t.first + tile_slot(false, lane, e));
         } else {
 #pragma unroll
             for (int e = 0; e < kPerThread; ++e) {
@@ -158,19 +162,19 @@ gbuffer_kernel(const MapDev m, const GBufDev g, float *__restrict__ sil, float *
             load(tn, dn);                  // next tile's loads fly during this tile
         }
         LaneCoords c;
-        // the vector path's two pairs of pixels: one division for the first
-        // pixel, then steps of 1 and 63 along the row (one wrap at most in a
+        // a vector tile's pixels: one division for the first, then steps of 1
+        // and 63 (two pairs) or of 32 along the row (one wrap at most in a
         // buffer at least 64 pixels wide)
         const bool steps = t.vec && g.width >= 64;
         int px = 0, py = 0;
         if (steps)
-            pixel_of(g, t.first + tile_slot(true, lane, 0), px, py);
+            pixel_of(g, t.first + tile_slot(TEX != 0, lane, 0), px, py);
 #pragma unroll
         for (int e = 0; e < kPerThread; ++e) {
-            const long long f = t.first + tile_slot(t.vec, lane, e);
+            const long long f = t.first + tile_slot(TEX != 0 && t.vec, lane, e);
             c.x[e] = c.y[e] = c.z[e] = 0.0f;
             if (steps) {
-                if (e > 0 && (px += e == 2 ? 63 : 1) >= g.width) {
+                if (e > 0 && (px += TEX == 0 ? 32 : e == 2 ? 63 : 1) >= g.width) {
                     px -= g.width;
                     ++py;
                 }
@@ -181,7 +185,7 @@ gbuffer_kernel(const MapDev m, const GBufDev g, float *__restrict__ sil, float *
                 project(g.m, qx, qy, d[e], c.x[e], c.y[e], c.z[e]);
             }
         }
-        classify_warp_tile<MODE, CODES>(m, t, c, wq[warp], queued);
+        classify_warp_tile<MODE, CODES, TEX>(m, t, c, wq[warp], queued);
         drain(queued, false);
         if (!more)
             break;
@@ -194,14 +198,14 @@ gbuffer_kernel(const MapDev m, const GBufDev g, float *__restrict__ sil, float *
     drain(queued, true);
 }
 
-template <int MODE, bool CODES>
+template <int MODE, bool CODES, int TEX>
 int launch_gbuffer(const MapDev &map, const GBufDev &g, float *sil, float *fil, uint16_t *codes, bool vec,
                    int max_dist, bool overlap, cudaStream_t stream)
 {
     // two CTAs of 20 warps per SM at 48 registers: 201 us for 4 frames of
     // 3840x2160 pixels, against 213 with four of 8 warps at 64 registers
     constexpr int kThreads = 640;
-    auto kern = gbuffer_kernel<MODE, CODES, kThreads>;
+    auto kern = gbuffer_kernel<MODE, CODES, kThreads, TEX>;
     static KernelSetup setup;
     int occupancy = 0;
     int rc = setup.get(kern, kThreads, 0, &occupancy);
@@ -240,6 +244,14 @@ int launch_gbuffer(const MapDev &map, const GBufDev &g, float *sil, float *fil, 
     if (e != cudaSuccess)
         return cuda_fail(e);
     return RBSM_OK;
+}
+
+template <int MODE, bool CODES>
+int launch_gbuffer(const MapDev &map, const GBufDev &g, float *sil, float *fil, uint16_t *codes, bool vec,
+                   int max_dist, bool overlap, cudaStream_t stream)
+{
+    return map.tex ? launch_gbuffer<MODE, CODES, 1>(map, g, sil, fil, codes, vec, max_dist, overlap, stream)
+                   : launch_gbuffer<MODE, CODES, 0>(map, g, sil, fil, codes, vec, max_dist, overlap, stream);
 }
 
 struct Span {

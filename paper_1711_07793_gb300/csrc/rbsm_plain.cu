@@ -91,7 +91,7 @@ struct PlainJobs {
 // take the tiles after it.  (A fixed share for each warp: 60.8 against 54.1 us
 // on 3840x2160 fragments, filtering, with CTAs of 8 warps.)  The next tile
 // waits in shared memory (cp.async), not in registers.
-template <int MODE, bool CODES, int kThreads>
+template <int MODE, bool CODES, int kThreads, int TEX>
 __global__ void __launch_bounds__(kThreads, kThreads == 1024 ? 1 : 1280 / kThreads)
 plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restrict__ y,
              const float *__restrict__ z, long long n, float *__restrict__ sil,
@@ -143,12 +143,12 @@ plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restric
         const bool more = nt < tiles;
         WarpTileIO tn;
         LaneCoords c;
-        fetch_tile(t, lane, buf, c);
+        fetch_tile<TEX == 0>(t, lane, buf, c);
         if (more) {
             tn = io_of(nt);
             stage_tile(tn, lane, buf);     // next tile's copies fly during this tile
         }
-        classify_warp_tile<MODE, CODES>(m, t, c, wq[warp], queued);
+        classify_warp_tile<MODE, CODES, TEX>(m, t, c, wq[warp], queued);
         drain_queue<PlainJobs, MODE, kThreads == 1024>(jobs, wq[warp], queued, max_dist, false);
         if (!more)
             break;
@@ -166,11 +166,11 @@ plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restric
 // 49.2 / 20.2 now).
 bool plain_large(int64_t n, int sms) { return (n + kWarpTile - 1) / kWarpTile >= 32LL * sms; }
 
-template <int MODE, bool CODES, int kThreads>
+template <int MODE, bool CODES, int kThreads, int TEX>
 int launch_plain(const rbsm_map &map, const rbsm_frags &f, float *sil, float *fil, uint16_t *codes,
                  int max_dist, int sms, cudaStream_t stream)
 {
-    auto kern = plain_kernel<MODE, CODES, kThreads>;
+    auto kern = plain_kernel<MODE, CODES, kThreads, TEX>;
     static KernelSetup setup;
     int occupancy = 0;
     int rc = setup.get(kern, kThreads, 0, &occupancy);
@@ -200,9 +200,11 @@ int launch_plain(const rbsm_map &map, const rbsm_frags &f, float *sil, float *fi
     const int sms = device_sm_count();
     if (sms <= 0)
         return cuda_fail(cudaErrorNoDevice);
-    return plain_large(f.n, sms)
-               ? launch_plain<MODE, CODES, 1024>(map, f, sil, fil, codes, max_dist, sms, stream)
-               : launch_plain<MODE, CODES, 256>(map, f, sil, fil, codes, max_dist, sms, stream);
+    if (plain_large(f.n, sms))
+        return map.texture ? launch_plain<MODE, CODES, 1024, 1>(map, f, sil, fil, codes, max_dist, sms, stream)
+                           : launch_plain<MODE, CODES, 1024, 0>(map, f, sil, fil, codes, max_dist, sms, stream);
+    return map.texture ? launch_plain<MODE, CODES, 256, 1>(map, f, sil, fil, codes, max_dist, sms, stream)
+                       : launch_plain<MODE, CODES, 256, 0>(map, f, sil, fil, codes, max_dist, sms, stream);
 }
 
 bool overlaps_inputs(const rbsm_map &m, const rbsm_frags &f, const void *out, size_t bytes)
