@@ -18,7 +18,7 @@
 // edge samples writes its mean at once, and one outside the shared block
 // (below) walks its own samples, so no second pass is needed.  For k = 1
 // there is nothing to add and the answers are stored as floats
-// (rsmss_filter's bits, and its kernel on large textured calls).  Because the answers do not depend on the order of
+// (rsmss_filter's bits, and its kernel on large calls).  Because the answers do not depend on the order of
 // the work, the warps of a CTA share its strips as they come free.
 #include <cuda_runtime.h>
 
@@ -518,12 +518,11 @@ int rpcf_entry(const rbsm_map *map, const rbsm_frags *frags, float *vis, int32_t
                 reinterpret_cast<uintptr_t>(vis) < reinterpret_cast<uintptr_t>(ws) + 8u)))
         return RBSM_ERR_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // k = 1 is rsmss_filter: with a texture and enough tiles for CTAs of 1024
-    // its kernel (3840x2160 / 1277x719 fragments 47.0 / 14.9 against 57.6 /
-    // 16.5 us here); without one, or on few fragments, one strip per warp
-    // finishes sooner (3840x2160 without a texture 76.1 against 80.2 us, one
-    // call on 320x240 22.3 against 25.7)
-    if (k == 1 && map->texture && plain_large(frags->n, device_sm_count()))
+    // k = 1 is rsmss_filter: with tiles enough for CTAs of 1024 its kernel
+    // (3840x2160 / 1277x719 fragments 47.0 / 14.9 against 57.6 / 16.5 us here;
+    // 3840x2160 without a texture 66.6 against 75.8); on few fragments one strip
+    // per warp finishes sooner (one call on 320x240 22.3 against 25.7)
+    if (k == 1 && plain_large(frags->n, device_sm_count()))
         return plain_entry(RBSM_MODE_FILTER, map, frags, vis, nullptr, params, stream);
     switch (k) {
     case 1: return launch_rpcf<1>(*map, *frags, vis, max_dist, s);
