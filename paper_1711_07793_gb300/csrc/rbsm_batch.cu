@@ -65,6 +65,8 @@ int occupancy_of(BatchKernelFn fn, int threads, size_t smem, int *occ)
 template <int kThreads, bool LEARNED, int kMinBlocks>
 BatchKernelFn kernel_for(int umode)
 {
+    if (umode > 6)
+        return batch_kernel_untextured(LEARNED, umode);
     if (kThreads == 256 && kMinBlocks == 4)
         return batch_kernel_256_4(LEARNED, umode);
     if (kThreads == 256 && kMinBlocks == 3)
@@ -120,6 +122,28 @@ int uniform_mode(const BatchArgs &a)
     return 2 * m + c - 1;
 }
 
+// Whether a batch of one (mode, codes) pair takes the kernels for maps
+// without textures (UMODE + 6): no map it samples has one, and most of its
+// fragments sample maps of at least twice as many texels as the job has
+// fragments.  There single fragments 32 apart touch half the lines a pair
+// does (8 frames of 3840x2160 on 8192^2 maps 583 -> 495 us, one 91 -> 80);
+// fragments that share texels are served by either, and the pairs cost fewer
+// accesses to shared memory (64 cascade jobs, half of them on maps of fewer
+// texels than fragments: 417 us with pairs, 423 with single ones).
+bool untextured(const BatchArgs &a)
+{
+    long long all = 0, wide = 0;
+    for (int k = 0; k < a.n_jobs; ++k) {
+        const MapDev &m = a.maps[a.jobs[k].map];
+        if (m.tex)
+            return false;
+        all += a.jobs[k].n;
+        if ((long long)m.width * m.height >= 2 * a.jobs[k].n)
+            wide += a.jobs[k].n;
+    }
+    return 4 * wide >= 3 * all;
+}
+
 // Kernel variant for a launch request.  At 256 threads the exact path has
 // variants with registers sized for 3, 4 and 5 CTAs per SM (80, 64, 48 per
 // thread): asking for 3 selects the first, 5 or the occupancy limit (0) the
@@ -131,11 +155,12 @@ int launch_shape(const BatchArgs &args, int threads, int ctas_per_sm, int chunk,
         return RBSM_ERR_ARG;
     const bool learned = args.mlp != nullptr;
     const int um = uniform_mode(args);
+    const int um_tex = um && untextured(args) ? um + 6 : um;
     if (learned) {
         switch (threads) {
         case 128: return shape_for<128, true, 8>(args, ctas_per_sm, chunk, 0, out);
         case 512: return shape_for<512, true, 2>(args, ctas_per_sm, chunk, 0, out);
-        default: return shape_for<256, true, 4>(args, ctas_per_sm, chunk, um, out);
+        default: return shape_for<256, true, 4>(args, ctas_per_sm, chunk, um == 3 || um == 4 ? um_tex : um, out);
         }
     }
     switch (threads) {
@@ -144,7 +169,7 @@ int launch_shape(const BatchArgs &args, int threads, int ctas_per_sm, int chunk,
     default:
         if (ctas_per_sm == 3) return shape_for<256, false, 3>(args, ctas_per_sm, chunk, um, out);
         if (ctas_per_sm == 0 || ctas_per_sm >= 5)
-            return shape_for<256, false, 5>(args, ctas_per_sm, chunk, um, out);
+            return shape_for<256, false, 5>(args, ctas_per_sm, chunk, um_tex, out);
         return shape_for<256, false, 4>(args, ctas_per_sm, chunk, um, out);
     }
 }

@@ -260,12 +260,15 @@ constexpr size_t batch_smem_bytes()
 // UMODE 0: each job's mode and codes flag are read at run time; UMODE
 // 2 * mode + codes - 1 (1..6): every job of the launch has that pair, which
 // keeps one specialisation of the classification in the loop (the run-time
-// dispatch inlines all six and costs registers).
+// dispatch inlines all six and costs registers); UMODE 7..12: the same
+// pairs, and no map has a texture (kernels of classify_warp_tile's TEX 0).
 template <int kThreads, bool LEARNED, int kMinBlocks, int UMODE>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) batch_kernel(const __grid_constant__ BatchArgs a)
 {
-    constexpr int kFixedMode = (UMODE + 1) / 2;
-    constexpr bool kFixedCodes = ((UMODE + 1) % 2) == 1;
+    constexpr int kPair = UMODE > 6 ? UMODE - 6 : UMODE;
+    constexpr int kTex = UMODE > 6 ? 0 : -1;
+    constexpr int kFixedMode = (kPair + 1) / 2;
+    constexpr bool kFixedCodes = ((kPair + 1) % 2) == 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     auto &bs = *reinterpret_cast<BatchSmem<kThreads, LEARNED> *>(smem_raw);
     auto &ls = *reinterpret_cast<LearnedSmem<kThreads> *>(smem_raw + sizeof(BatchSmem<kThreads, LEARNED>));
@@ -366,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) batch_kernel(const __gri
         int njob = job;
         WarpTileIO tn;
         LaneCoords c;
-        fetch_tile(t, lane, buf, c);
+        fetch_tile<kTex == 0>(t, lane, buf, c);
         if (more) {
             if (nt < job_lo || nt >= job_hi) {
                 // mostly a few jobs on (the claims advance through the list)
@@ -392,8 +395,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) batch_kernel(const __gri
         if (UMODE == 0)
             classify_warp_tile_rt(J.mode, J.codes_on != 0, kCopyMap ? map : a.maps[J.map], t, c, wq, queued);
         else
-            classify_warp_tile<kFixedMode ? kFixedMode : 1, kFixedCodes>(kCopyMap ? map : a.maps[J.map], t, c, wq,
-                                                                         queued);
+            classify_warp_tile<kFixedMode ? kFixedMode : 1, kFixedCodes, kTex>(kCopyMap ? map : a.maps[J.map], t, c,
+                                                                               wq, queued);
         if (LEARNED)
             drain_queue_learned<BatchJobs, kThreads>(jobs, wq, queued, candidates, a.max_dist, false, ls, warp, a.tau,
                                                      a.stats);
@@ -421,5 +424,6 @@ BatchKernelFn batch_kernel_256_4(bool learned, int umode);
 BatchKernelFn batch_kernel_256_3(int umode);
 BatchKernelFn batch_kernel_256_5(int umode);
 BatchKernelFn batch_kernel_misc(int threads, bool learned);
+BatchKernelFn batch_kernel_untextured(bool learned, int umode);      // 7..12; learned: 9, 10
 
 }  // namespace rbsm

@@ -53,3 +53,21 @@ def test_depth_buffers(scene, w, mode):
         assert torch.equal(a.vis_silhouette, b.vis_silhouette)
     if mode & 2:
         assert torch.equal(a.vis_filter, b.vis_filter)
+
+
+@pytest.mark.parametrize("codes", [False, True])
+@pytest.mark.parametrize("mode", [1, 2, 3])
+def test_batches(scene, mode, codes):
+    """Jobs of fewer and of more fragments than half the map's texels (24960): the line between the kernels."""
+    api, g, depth, tex = scene
+    for sizes in ([12480, 129], [12481, 31], [40000, 5000, 127]):
+        xyz = [[torch.rand(n, generator=g, device="cuda") * 1.04 - 0.02 for _ in range(3)] for n in sizes]
+        runs = []
+        for m in (depth, tex):
+            batch = api.Batch([m], [api.Job(0, *p, mode=mode, codes=codes or None) for p in xyz])
+            api.rbsm_batch_run(batch)
+            runs.append(batch.jobs)
+        for a, b in zip(*runs):
+            for k in ("vis_silhouette", "vis_filter", "codes"):
+                assert (getattr(a, k) is None) == (getattr(b, k) is None)
+                assert getattr(a, k) is None or torch.equal(getattr(a, k), getattr(b, k))
