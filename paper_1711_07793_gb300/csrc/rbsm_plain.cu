@@ -200,6 +200,7 @@ int launch_plain(const rbsm_map &map, const rbsm_frags &f, float *sil, float *fi
     const int sms = device_sm_count();
     if (sms <= 0)
         return cuda_fail(cudaErrorNoDevice);
+    // a kernel for each kind of map (classify_warp_tile has the figures)
     if (plain_large(f.n, sms))
         return map.texture ? launch_plain<MODE, CODES, 1024, 1>(map, f, sil, fil, codes, max_dist, sms, stream)
                            : launch_plain<MODE, CODES, 1024, 0>(map, f, sil, fil, codes, max_dist, sms, stream);
