@@ -548,9 +548,12 @@ __device__ __forceinline__ void stage_tile(const WarpTileIO &t, unsigned lane, f
 // that copied it: a warp barrier after the wait, and another before it is
 // refilled.
 //
-// SINGLES: single fragments 32 apart, for kernels that read a map without a
+// SINGLES: single fragments 32 apart.  For kernels that read a map without a
 // texture: each of a fragment's five loads then covers 32 fragments in a row
-// and touches half the lines.
+// and touches half the lines.  And for the single-map calls, whose answers
+// are one plane (filtering 3840x2160 47.7 us with pairs, 47.2 with singles;
+// 2560x1440 29.5 and 28.6; silhouette 1920x1080 20.3 and 19.8).  Depth buffers with two answer planes keep the pairs
+// (194.7 against 197.9 us for 4 frames).
 template <bool SINGLES = false>
 __device__ __forceinline__ void fetch_tile(const WarpTileIO &t, unsigned lane, const float4 (&buf)[3][32],
                                            LaneCoords &c)
@@ -626,18 +629,17 @@ __device__ __forceinline__ void drain_queue(const Jobs &jobs, WarpQueue &wq, int
 // Classify one warp tile whose coordinates the lane holds, store its answers
 // (provisional for edge fragments) and queue its edge fragments.  TEX: whether
 // the map has a texture, 1 or 0, or -1 to ask the map per tile.  Kernels
-// made for one of them hold half the code, and without a texture (0) a
-// lane's fragments are single ones 32 apart (see fetch_tile; -1 keeps the
-// pairs).  3840x2160 fragments without a texture: filtering 75.2 us with pairs
+// made for one of them hold half the code.  PAIRS: a lane's fragments in a
+// vector tile are two pairs, else single ones 32 apart (see fetch_tile).  3840x2160 fragments without a texture: filtering 75.2 us with pairs
 // and a kernel for both, 56.4 with TEX 0; silhouette 67.4 and 53.0; depth
 // buffers, 4 frames, 313 and 266 (with a texture 195.4 and 193.4, TEX 1).
-template <int MODE, bool CODES, int TEX = -1>
+template <int MODE, bool CODES, int TEX = -1, bool PAIRS = TEX != 0>
 __device__ __forceinline__ void classify_warp_tile(const MapDev &m, const WarpTileIO &t, const LaneCoords &c,
                                                    WarpQueue &wq, int &count)
 {
     const unsigned lane = lane_id();
     const unsigned below = (1u << lane) - 1u;
-    const bool pairs = TEX != 0 && t.vec;
+    const bool pairs = PAIRS && t.vec;
     FragResult r[kPerThread];
     uint32_t bits[kPerThread];
     bool edge[kPerThread];

@@ -143,12 +143,12 @@ plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restric
         const bool more = nt < tiles;
         WarpTileIO tn;
         LaneCoords c;
-        fetch_tile<TEX == 0>(t, lane, buf, c);
+        fetch_tile<true>(t, lane, buf, c);
         if (more) {
             tn = io_of(nt);
             stage_tile(tn, lane, buf);     // next tile's copies fly during this tile
         }
-        classify_warp_tile<MODE, CODES, TEX>(m, t, c, wq[warp], queued);
+        classify_warp_tile<MODE, CODES, TEX, false>(m, t, c, wq[warp], queued);
         drain_queue<PlainJobs, MODE, kThreads == 1024>(jobs, wq[warp], queued, max_dist, false);
         if (!more)
             break;
@@ -163,7 +163,7 @@ plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restric
 // more SMs.  3840x2160 filtering / 1920x1080 silhouette: 52.5 / 22.4 us with
 // 1024, 53.1 / 23.0 with two of 640, 52.2 / 24.4 with four of 320, 54.3 / 23.3
 // with five of 256 (before the walks' pairs of steps and the runs of 16:
-// 49.2 / 20.2 now).
+// 49.2 / 20.2; 47.2 / 19.8 with single fragments 32 apart).
 bool plain_large(int64_t n, int sms) { return (n + kWarpTile - 1) / kWarpTile >= 32LL * sms; }
 
 template <int MODE, bool CODES, int kThreads, int TEX>
