@@ -5,6 +5,7 @@ else.  There is no fallback: when librbsm.so is missing or cannot be loaded,
 ``lib()`` raises, so nothing can silently run a different implementation.
 """
 import ctypes
+import hashlib
 import os
 import re
 
@@ -113,6 +114,7 @@ class RBSMError(RuntimeError):
 
 
 _lib = None
+_fingerprint = None
 _P = ctypes.POINTER
 
 
@@ -199,15 +201,25 @@ def _declare(lib):
 
 def lib():
     """The loaded librbsm.so (raises when it has not been built)."""
-    global _lib
+    global _lib, _fingerprint
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError("librbsm.so is not built (%s); run paper_1711_07793_gb300.build.build()"
                                % LIB_PATH)
+        with open(LIB_PATH, "rb") as f:
+            digest = hashlib.sha256(f.read()).hexdigest()[:16]
         l = ctypes.CDLL(LIB_PATH)
         _declare(l)
+        _fingerprint = digest
         _lib = l
     return _lib
+
+
+def library_fingerprint():
+    """Digest of the loaded librbsm.so (taken when it was loaded): what was
+    measured with one build of the kernels is not applied to another."""
+    lib()
+    return _fingerprint
 
 
 def status_string(code):

@@ -277,11 +277,14 @@ class BatchGraph:
 
 
 def batch_signature(batch):
-    """Key of a batch for the autotuner cache: device, map sizes, job sizes."""
+    """Key of a batch for the autotuner cache: the library's build, device,
+    map sizes, job sizes.  (A pick is a timing of one build's kernels: with
+    the build left out, a launch shape picked for kernels that have since been
+    rewritten would be applied unseen.)"""
     name = torch.cuda.get_device_name(batch.jobs[0].x.device)
     maps = [tuple(m.depth.shape) + ("tex",) if isinstance(m, MapTexture) else tuple(m.shape) for m in batch.maps]
     jobs = [(j.map_index, j.mode, int(j.x.shape[0]), j.codes is not None) for j in batch.jobs]
-    return json.dumps(["v2", name, maps, jobs])
+    return json.dumps(["v3", N.library_fingerprint(), name, maps, jobs])
 
 
 TUNE_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "autotune_cache.json")
