@@ -31,14 +31,15 @@
 
 #include "rbsm.h"
 #include "rbsm_host.h"
+#include "rbsm_rules.h"
 
 namespace rbsm {
 namespace {
 
 constexpr int kSmThreads = 256;           // 8 warps
-constexpr int kLargeTile = 64;            // texels per tile side on large maps
 constexpr int kBlockRows = 4;             // a warp works on blocks of 32 x 4 texels
 constexpr int kChunk = kSmThreads;        // occluders culled per round
+static_assert(kChunk == kLightRound, "the tile rule counts one culling round");
 constexpr float kCullSlack = 0.5f;        // texels added to every (float) culling bound
 
 // A surviving occluder of the current tile: its position relative to the tile
@@ -88,7 +89,7 @@ struct TileSmem {
 // CTA, for the culling and the float pre-tests; `ea` bounds what the
 // rounding of the centre to float moves any projection (|c - c_f| (|ux| +
 // |uy|) <= (|cx| + |cy|) 2^-24 * sqrt 2, taken as 2^-22).
-constexpr int kFloatCopies = 256;
+constexpr int kFloatCopies = kLightRound;
 struct FloatOcc {
     float cx, cy, ux, uy, ha, hb, ea, depth;
 };
@@ -591,8 +592,11 @@ int launch_map(const rbsm_occluders &occ, float *depth, int width, int height, l
     const int sms = device_sm_count();
     if (sms <= 0)
         return cuda_fail(cudaErrorNoDevice);
-    auto tiles_of = [&](long long side) { return ((width + side - 1) / side) * ((height + side - 1) / side); };
-    const bool large = copies && (long long)occ.n_rects + occ.n_spheres <= kChunk && tiles_of(kLargeTile) >= 2LL * 4 * sms;
+    // 1 / zscale as a pair of floats, for scales of 2^-100 to 2^100
+    const double inv_any = 1.0 / occ.zscale;
+    const bool fast = inv_any >= 7.888609052210118e-31 && inv_any <= 1.2676506002282294e30;
+    const float hi = fast ? (float)inv_any : 0.0f, lo = fast ? (float)(inv_any - (double)hi) : 0.0f;
+    const bool large = light_large_tiles(width, height, occ.n_rects, occ.n_spheres, fast, sms);
     static KernelSetup setup[3];
     const int which = large ? 2 : copies ? 1 : 0;
     auto kern = large ? shadow_map_kernel<true, kLargeTile> : copies ? shadow_map_kernel<true, 32> : shadow_map_kernel<false, 32>;
@@ -600,16 +604,12 @@ int launch_map(const rbsm_occluders &occ, float *depth, int width, int height, l
     int rc = setup[which].get(kern, kSmThreads, 0, &occupancy);
     if (rc != RBSM_OK)
         return rc;
-    const long long tiles = tiles_of(large ? kLargeTile : 32);
+    const long long tiles = square_tiles(width, height, large ? kLargeTile : 32);
     long long grid = (long long)sms * occupancy;
     if (grid > tiles)
         grid = tiles;
     int e2 = 0;
     const double inv = std::frexp(occ.zscale, &e2) == 0.5 ? std::ldexp(1.0, 1 - e2) : 0.0;
-    // 1 / zscale as a pair of floats, for scales of 2^-100 to 2^100
-    const double inv_any = 1.0 / occ.zscale;
-    const bool fast = inv_any >= 7.888609052210118e-31 && inv_any <= 1.2676506002282294e30;
-    const float hi = fast ? (float)inv_any : 0.0f, lo = fast ? (float)(inv_any - (double)hi) : 0.0f;
     cudaError_t e;
     if (overlap) {
         cudaLaunchConfig_t cfg = {};
