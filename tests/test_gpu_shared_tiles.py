@@ -2,13 +2,17 @@
 depth buffers, RPCF): a fragment's answer does not depend on how many
 fragments follow it, so the answers of n fragments are the first n of a larger
 call's, bit for bit, for n around the strips, runs, CTA shapes and waves the
-launches switch at; and nothing past the last fragment is written."""
+launches switch at; and nothing past the last fragment is written.  The map
+holds runs and one-texel lines, so that the walks end at every step up to the
+cap: small and large calls take them one and two steps at a time."""
 import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 
 pytestmark = pytest.mark.gpu
+
+from tests.test_gpu_walks import _map  # noqa: E402
 
 
 @pytest.fixture(scope="module")
@@ -20,7 +24,7 @@ def scene():
     from paper_1711_07793_gb300 import api
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     g = torch.Generator(device="cuda").manual_seed(3)
-    depth = torch.where(torch.rand((250, 384), generator=g, device="cuda") < 0.01, 0.3, 1.0)
+    depth = torch.from_numpy(_map(np.random.default_rng(3), 384, 250)).cuda()
     n = sms * 40 * 128 * 3 + 77
     x, y = (torch.rand(n, generator=g, device="cuda") * 1.02 - 0.01 for _ in range(2))
     return api, sms, depth, x, y, torch.full((n,), 0.75, device="cuda")

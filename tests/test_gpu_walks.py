@@ -3,7 +3,10 @@ of fragment (straight edge, corner, dead end, one-texel feature, lone texel)
 with walks that end, leave the edge, run into the border or into the cap, on
 maps down to one texel wide, against the oracle: codes and silhouette bit for
 bit, filtering within 1e-5 (one float32 add and divide per axis against the
-oracle's float64)."""
+oracle's float64).  Once with few fragments (CTAs of 256 threads, walks one
+step at a time) and once with the same fragments repeated until the single-map
+calls take their CTAs of 1024 threads, whose walks go two steps at a time past
+the second."""
 import numpy as np
 import pytest
 
@@ -29,10 +32,13 @@ def _map(rng, w, h):
     return m
 
 
-@pytest.mark.parametrize("max_dist", [1, 2, 3, 16, 255])
-@pytest.mark.parametrize("size", [(1, 1), (1, 40), (40, 1), (2, 3), (33, 29), (64, 48), (300, 5)])
-@pytest.mark.parametrize("texture", [False, True])
-def test_walks_match_the_oracle(size, max_dist, texture):
+CAPS = pytest.mark.parametrize("max_dist", [1, 2, 3, 16, 255])
+SIZES = pytest.mark.parametrize("size", [(1, 1), (1, 40), (40, 1), (2, 3), (33, 29), (64, 48), (300, 5)])
+TEXTURES = pytest.mark.parametrize("texture", [False, True])
+
+
+def _case(size, max_dist, texture):
+    """(api, map, map on the GPU, fragments)."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     import __graft_entry__
@@ -53,8 +59,36 @@ def test_walks_match_the_oracle(size, max_dist, texture):
         depth = api.MapTexture(pitched)
     else:
         depth = dev(m)
+    return api, m, depth, (x, y, z)
+
+
+@CAPS
+@SIZES
+@TEXTURES
+def test_walks_match_the_oracle(size, max_dist, texture):
+    api, m, depth, (x, y, z) = _case(size, max_dist, texture)
     for fn, mode in ((api.rbsm_visibility, orc.MODE_SILHOUETTE), (api.rsmss_filter, orc.MODE_FILTER)):
         vis, codes = fn(depth, dev(x), dev(y), dev(z), codes=True, max_dist=max_dist)
         torch.cuda.synchronize()
         ref = orc.evaluate(m, x, y, z, mode, max_dist=max_dist)
         assert_parity(vis.cpu().numpy(), codes.cpu().numpy().view(np.uint16), ref, mode, "%s %d" % (size, max_dist))
+
+
+@CAPS
+@SIZES
+@TEXTURES
+def test_walks_of_large_calls_match_the_oracle(size, max_dist, texture):
+    api, m, depth, (x, y, z) = _case(size, max_dist, texture)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    times = 128 * 32 * sms // x.size + 1               # 32 tiles of 128 for every SM
+    n = times * x.size
+    xyz = [dev(a).repeat(times) for a in (x, y, z)]
+    for fn, mode in ((api.rbsm_visibility, orc.MODE_SILHOUETTE), (api.rsmss_filter, orc.MODE_FILTER)):
+        ref = orc.evaluate(m, x, y, z, mode, max_dist=max_dist)
+        vis, codes = fn(depth, *xyz, codes=True, max_dist=max_dist)
+        # every repetition is the first one, and the first one the oracle's
+        assert torch.equal(vis, vis[:x.size].repeat(times)) and torch.equal(codes, codes[:x.size].repeat(times))
+        assert_parity(vis[:x.size].cpu().numpy(), codes[:x.size].cpu().numpy().view(np.uint16), ref, mode,
+                      "%s %d, %d fragments" % (size, max_dist, n))
+        # the kernel that writes no codes
+        assert torch.equal(fn(depth, *xyz, codes=False, max_dist=max_dist)[0], vis)
