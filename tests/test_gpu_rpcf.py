@@ -199,10 +199,9 @@ def test_shared_block_at_the_maximum_extent(api, k):
 
 @pytest.mark.parametrize("k", [1, 3, 5, 7])
 def test_workspace_schedule_gives_the_same_bits(api, k):
-    """rbsm_rpcf_ws (tiles taken from a counter) against rbsm_rpcf (a fixed
-    partition): the same bits on C2 at a reduced view, on odd maps with
-    borders and non-finite coordinates, and twice in a row with one
-    workspace (the call zeroes its counter)."""
+    """rbsm_rpcf_ws against rbsm_rpcf: the same bits on C2 at a reduced view,
+    on odd maps with borders and non-finite coordinates, and twice in a row
+    with one workspace, which the call leaves alone."""
     import rbsm_scenes as sc
     f = sc.config2(5, screen=(960, 540))
     rng = np.random.default_rng(40 + k)
@@ -211,13 +210,14 @@ def test_workspace_schedule_gives_the_same_bits(api, k):
     oy = rng.uniform(-0.3, 1.3, 30000).astype(np.float32)
     ox[::97] = np.nan
     cases = [(f.depth, f.x, f.y, f.z), (odd, ox, oy, np.full_like(ox, 0.5))]
-    ws = torch.zeros(1, dtype=torch.int64, device="cuda")
+    ws = torch.full((1,), -5, dtype=torch.int64, device="cuda")
     for depth, x, y, z in cases:
         d, xs, ys, zs = dev(depth), dev(x), dev(y), dev(z)
         ref = api.rbsm_rpcf(d, xs, ys, zs, k=k, workspace=None)           # rbsm_rpcf
         for _ in range(2):
             got = api.rbsm_rpcf(d, xs, ys, zs, k=k, workspace=ws)
-            auto = api.rbsm_rpcf(d, xs, ys, zs, k=k)                     # the binding's per-stream counter
+            auto = api.rbsm_rpcf(d, xs, ys, zs, k=k)                     # the binding's default: rbsm_rpcf
             torch.cuda.synchronize()
             assert torch.equal(got.view(torch.int32), ref.view(torch.int32))
             assert torch.equal(auto.view(torch.int32), ref.view(torch.int32))
+    assert int(ws) == -5
