@@ -34,4 +34,21 @@ inline bool light_large_tiles(int width, int height, int64_t n_rects, int64_t n_
            square_tiles(width, height, kLargeTile) >= 2LL * 4 * sms;
 }
 
+// The light pass with tiles of 32: whether a thread's rows are spread over its
+// tile.  From 32 tiles on, up to two for each of four CTAs per SM, the time of
+// a map is that of its tiles' slowest warps, and spreading the rows beats turning
+// blocks down as a whole (us, spread / blocks, with 24 rectangles, with 140 and
+// 60 spheres and with 200 of each: 192^2 3.8 / 4.2, 10.6 / 10.6 and 15.9 / 16.4;
+// 256^2 3.5 / 3.6, 8.7 / 9.1 and 13.9 / 15.2; 512^2 3.9 / 4.3, 7.8 / 9.0 and 14.4
+// / 15.9; 768^2 4.3 / 4.4, 10.1 / 10.7 and 18.9 / 19.1; 1024^2 5.2 / 5.3, 12.6 / 13.3 and
+// 22.4 / 22.9).  On fewer tiles the occluders that fill a block count (128^2 3.8 /
+// 4.1, 14.0 / 12.0 and 23.2 / 21.0), and on more the work in all (2048^2 10.3 /
+// 10.6, 23.1 / 23.3 and 39.7 / 39.0; with 300 rectangles 41.3 / 38.0, with 200
+// large ones 117 / 79).
+inline bool light_spread_rows(int width, int height, int sms)
+{
+    const long long tiles = square_tiles(width, height, 32);
+    return tiles > 32 && tiles <= 8LL * sms;
+}
+
 }  // namespace rbsm

@@ -414,6 +414,11 @@ __device__ __forceinline__ void cull_round(const rbsm_occluders &occ, const Floa
 // kTile: texels per tile side, 32 (one block per warp) or a larger multiple
 // of 32 (several blocks per warp, and at most kChunk occluders in all).
 //
+// SPREAD (kTile 32): a thread's 4 rows are 8 apart, so that every warp works on
+// all of the tile's height, and no block is turned down as a whole.  For maps of
+// few tiles, which take as long as a tile's slowest warp (light_spread_rows has
+// the figures).
+//
 // Bound: instruction issue.  Culling a tile costs a warp about 270
 // instructions whatever the tile holds, so large maps take tiles of 64 and
 // the warps turn survivors down (or take a rectangle over the whole of a
@@ -422,7 +427,7 @@ __device__ __forceinline__ void cull_round(const rbsm_occluders &occ, const Floa
 // 128: 160; blocks handed to the warps one at a time: 163); the reciprocal
 // root, the FastTwoSums and the thresholds formed at the cull took the 150 to
 // 143.  One map's 268 MB take 40 us at the copy rate.
-template <bool COPIES, int kTile>
+template <bool COPIES, int kTile, bool SPREAD>
 __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_occluders occ, float *__restrict__ depth,
                                                                 int width, int height, long long pitch,
                                                                 double inv_zscale, float scale_hi, float scale_lo)
@@ -442,6 +447,8 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
     }
     const FloatOcc *fop = fo;
     const FloatSph *fsp = fs;
+    static_assert(!SPREAD || kTile == 32, "one block per warp");
+    constexpr int kRowStep = SPREAD ? kSmWarps : 1;       // between a thread's rows
     // 1 / zscale for the float-float cap depth: scale_hi + scale_lo, or no
     // float-float depths (scale_hi = 0: a scale out of its range)
     const bool fast = scale_hi > 0.0f;
@@ -467,35 +474,37 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
         }
         // tile centre (i0 + 0.5 + (kTile - 1) / 2, ...), exact (< 2^23)
         const float tcx = small_int_float(i0 + kTile / 2), tcy = small_int_float(j0 + kTile / 2);
-        // one block of 32 x 4 texels (this thread: a column of 4) against the
-        // survivors of a culling round
+        // one block of 32 x 4 texels (this thread: a column of 4, the rows bj +
+        // kRowStep p) against the survivors of a culling round
         auto test_block = [&](int bi, int bj, const Cand *buf, int nr, int ns, float (&best)[kBlockRows]) {
-            // block centre and this thread's texel centres - tile centre, exact
+            // block centre (of rows 1 apart) and this thread's texel centres - tile centre, exact
             const float bx = __fsub_rn(small_int_float(bi) + 15.5f, h), by = __fsub_rn(small_int_float(bj) + 1.5f, h);
             const float ox = __fsub_rn(small_int_float(bi + lane), h), oy0 = by - 1.5f;
             for (int q = 0; q < nr; ++q) {
                 const RectCand &r = buf[sm.idx[q]].r;
                 // the block against the rectangle
-                const float sb = fabsf(r.s0 + (bx * r.uxf + by * r.uyf)), tb = fabsf(r.t0 + (by * r.uxf - bx * r.uyf));
-                if (sb > r.bs_out || tb > r.bt_out)
-                    continue;                              // surely outside
-                if (sb < r.bs_in && tb < r.bt_in) {
+                if (!SPREAD) {
+                    const float sb = fabsf(r.s0 + (bx * r.uxf + by * r.uyf)), tb = fabsf(r.t0 + (by * r.uxf - bx * r.uyf));
+                    if (sb > r.bs_out || tb > r.bt_out)
+                        continue;                              // surely outside
+                    if (sb < r.bs_in && tb < r.bt_in) {
 #pragma unroll
-                    for (int p = 0; p < kBlockRows; ++p)   // surely covers the block
-                        best[p] = r.depth < best[p] ? r.depth : best[p];
-                    continue;
+                        for (int p = 0; p < kBlockRows; ++p)   // surely covers the block
+                            best[p] = r.depth < best[p] ? r.depth : best[p];
+                        continue;
+                    }
                 }
                 const float sx = ox * r.uxf, tx_ = -ox * r.uyf;
 #pragma unroll
                 for (int p = 0; p < kBlockRows; ++p) {
-                    const float oy = oy0 + (float)p;
+                    const float oy = oy0 + (float)(kRowStep * p);
                     const float sf = fabsf(r.s0 + (sx + oy * r.uyf));
                     const float tf = fabsf(r.t0 + (tx_ + oy * r.uxf));
                     if (sf > r.s_out || tf > r.t_out || !(r.depth < best[p]))
                         continue;                          // surely outside, or it cannot lower the depth
                     bool in = sf < r.s_in && tf < r.t_in;
                     if (!in)
-                        in = rect_covers_exact(occ.rects + r.k, i0 + bi + lane, j0 + bj + p);     // near an edge
+                        in = rect_covers_exact(occ.rects + r.k, i0 + bi + lane, j0 + bj + kRowStep * p);     // near an edge
                     if (in)
                         best[p] = r.depth;
                 }
@@ -504,7 +513,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
                 const SphereCand &c = buf[sm.idx[nr + q]].s;
                 // the disc against the block's box of texel centres
                 const float gx = fmaxf(fabsf(c.dx0 + bx) - 15.5f, 0.0f), gy = fmaxf(fabsf(c.dy0 + by) - 1.5f, 0.0f);
-                if (gx * gx + gy * gy > c.rb_out)
+                if (!SPREAD && gx * gx + gy * gy > c.rb_out)
                     continue;                              // surely outside
                 const float dxf = c.dx0 + ox;
                 const CapColumn col = cap_column(c, ox);
@@ -519,7 +528,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
                         float d = 0.0f;
                         const int cap = c.k >= 0 ? cap_fast(c, col, oy, scale_hi, scale_lo, d) : -1;
                         if (cap < 0)
-                            d = cap_depth_exact(occ.spheres + (c.k >= 0 ? c.k : ~c.k), i0 + bi + lane, j0 + bj + p, inv_zscale, occ.zscale);
+                            d = cap_depth_exact(occ.spheres + (c.k >= 0 ? c.k : ~c.k), i0 + bi + lane, j0 + bj + kRowStep * p, inv_zscale, occ.zscale);
                         if (cap != 0 && d < best[0])
                             best[0] = d;
                     }
@@ -528,7 +537,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
                     best[1] = best[2];
                     best[2] = best[3];
                     best[3] = f;
-                    oy = __fadd_rn(oy, 1.0f);              // exact
+                    oy = __fadd_rn(oy, (float)kRowStep);   // exact
                 }
             }
         };
@@ -538,15 +547,16 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
             if (i < width) {
 #pragma unroll
                 for (int p = 0; p < kBlockRows; ++p) {
-                    if (j + p < height)
+                    if (j + kRowStep * p < height)
                         *out = best[p];
-                    out += pitch;
+                    out += kRowStep * pitch;
                 }
             }
         };
         if (kTile == 32) {
             // one block per warp, against the occluders in rounds of kChunk:
             // rectangles, then spheres, in index order
+            const int bj = SPREAD ? warp : warp * kBlockRows;
             float best[kBlockRows];
 #pragma unroll
             for (int p = 0; p < kBlockRows; ++p)
@@ -555,9 +565,9 @@ __global__ void __launch_bounds__(kSmThreads, 4) shadow_map_kernel(const rbsm_oc
                 int nr, ns;
                 Cand *buf = sm.c[round++ & 1];
                 cull_round<COPIES, kTile>(occ, fop, fsp, base, tcx, tcy, fast, sm, buf, nr, ns);
-                test_block(0, warp * kBlockRows, buf, nr, ns, best);
+                test_block(0, bj, buf, nr, ns, best);
             }
-            store_block(0, warp * kBlockRows, best);
+            store_block(0, bj, best);
         } else {
             // one round of occluders (at most kChunk), then block after block
             int nr = 0, ns = 0;
@@ -597,9 +607,12 @@ int launch_map(const rbsm_occluders &occ, float *depth, int width, int height, l
     const bool fast = inv_any >= 7.888609052210118e-31 && inv_any <= 1.2676506002282294e30;
     const float hi = fast ? (float)inv_any : 0.0f, lo = fast ? (float)(inv_any - (double)hi) : 0.0f;
     const bool large = light_large_tiles(width, height, occ.n_rects, occ.n_spheres, fast, sms);
-    static KernelSetup setup[3];
-    const int which = large ? 2 : copies ? 1 : 0;
-    auto kern = large ? shadow_map_kernel<true, kLargeTile> : copies ? shadow_map_kernel<true, 32> : shadow_map_kernel<false, 32>;
+    const bool spread = !large && light_spread_rows(width, height, sms);
+    static KernelSetup setup[5];
+    const int which = large ? 4 : 2 * copies + spread;
+    auto kern = large    ? shadow_map_kernel<true, kLargeTile, false>
+                : copies ? (spread ? shadow_map_kernel<true, 32, true> : shadow_map_kernel<true, 32, false>)
+                         : (spread ? shadow_map_kernel<false, 32, true> : shadow_map_kernel<false, 32, false>);
     int occupancy = 0;
     int rc = setup[which].get(kern, kSmThreads, 0, &occupancy);
     if (rc != RBSM_OK)

@@ -1,9 +1,10 @@
-"""GPU test of the light pass's tiles of 64 texels (maps of at least two such
-tiles per resident CTA): odd sizes whose last tiles are partial, thin and wide
+"""GPU test of the light pass's forms: tiles of 64 texels (maps of at least two
+such tiles per resident CTA), and tiles of 32 with the warps on blocks of rows or
+on rows spread over the tile, on both sides of the lines between them.  Odd sizes whose last tiles are partial, thin and wide
 rectangles (blocks surely outside, surely covered, and cut), spheres from
-sub-texel to several tiles, depth scales that are powers of two and not, more
-occluders than one culling round (which keeps the small tiles), and a pitched
-output; bit for bit the brute-force oracle."""
+sub-texel to several tiles, depth scales that are powers of two and not or
+outside the float-float range, no occluders, more than one culling round of them
+(which keeps the small tiles), and a pitched output; bit for bit the brute-force oracle."""
 import numpy as np
 import pytest
 
@@ -30,8 +31,14 @@ def _occluders(rng, w, h, nr, ns):
 @pytest.mark.parametrize("w,h,nr,ns,zs", [(2305, 2241, 40, 25, 2048.0), (2305, 2241, 40, 25, 1000.0),
                                           (2240, 2240, 30, 30, 3.7), (2400, 2200, 0, 40, 0.3),
                                           (2400, 2200, 256, 0, 64.0), (2305, 2241, 250, 20, 777.7),
-                                          (9000, 577, 30, 30, 1e3)])
-def test_large_maps(w, h, nr, ns, zs):
+                                          (9000, 577, 30, 30, 1e3), (2305, 2241, 0, 0, 64.0),
+                                          (2305, 2241, 10, 12, 2.0 ** 101),
+                                          (160, 192, 20, 10, 64.0), (161, 192, 20, 10, 64.0), (161, 200, 200, 200, 3.0),
+                                          (500, 333, 120, 60, 512.0), (500, 333, 300, 290, 77.7),
+                                          (777, 768, 30, 20, 1000.0), (1, 1100, 12, 6, 2.0), (1089, 1120, 30, 20, 8.0),
+                                          (1121, 1120, 30, 20, 8.0),
+                                          (801, 800, 10, 300, 0.3)])
+def test_maps(w, h, nr, ns, zs):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     import __graft_entry__

@@ -40,3 +40,10 @@ def rule(tmp_path_factory):
 def test_light_pass_tiles(rule, size, rects, spheres, scale_in_range, large):
     assert rule("light_large_tiles(%d, %d, %d, %d, %s, %d)"
                 % (size, size, rects, spheres, str(scale_in_range).lower(), SMS)) == large
+
+
+@pytest.mark.parametrize("w,h,spread", [(128, 128, False), (160, 192, False), (192, 192, True), (512, 512, True),
+                                        (1024, 1024, True), (1216 * 32, 32, True), (1216 * 32 + 1, 32, False),
+                                        (2048, 2048, False)])
+def test_light_pass_rows(rule, w, h, spread):
+    assert rule("light_spread_rows(%d, %d, %d)" % (w, h, SMS)) == spread
