@@ -671,11 +671,15 @@ __device__ __forceinline__ void classify_warp_tile(const MapDev &m, const WarpTi
         }
     } else if (TEX == 0) {
         // the four fragments' own texels first, then their neighbours, so
-        // that no fragment's loads wait for another's (in silhouette recovery
-        // too, where a shadowed fragment needs none: 1920x1080 20.8 us,
-        // 3840x2160 53.0; branched past when shadowed 21.3 and 53.0, and one
-        // fragment after the other 22.3 and 59.2).  A partial tile's lanes
-        // past its end hold zeros and are masked after.
+        // that no fragment's loads wait for another's.  In silhouette recovery
+        // a shadowed fragment needs no neighbours, and its lane loads none: a view
+        // whose fragments run across the map's rows touches a line of its own
+        // with every load (2828x2828 fragments on a 4096^2 map, rows of
+        // fragments along its columns: all shadowed 42.7 us, half 151, lit 142;
+        // with the neighbours loaded in any case 116, 185 and 141; a 1920x1080
+        // view of a scene 21.5 and 20.9; one fragment after the other 61 us for
+        // 8 M lit fragments in order, where this takes 38).  A partial tile's
+        // lanes past its end hold zeros and are masked after.
         const float *p[kPerThread];
         float zc[kPerThread];
         int i[kPerThread], j[kPerThread];
@@ -690,6 +694,9 @@ __device__ __forceinline__ void classify_warp_tile(const MapDev &m, const WarpTi
         float4 nb[kPerThread];
 #pragma unroll
         for (int e = 0; e < kPerThread; ++e) {
+            nb[e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (MODE == 1 && !CODES && c.z[e] > zc[e])
+                continue;                      // classify_from asks for no neighbour
             nb[e].x = __ldg(p[e] - (i[e] > 0 ? 1 : 0));
             nb[e].y = __ldg(p[e] + (i[e] < m.width - 1 ? 1 : 0));
             nb[e].z = __ldg(p[e] + (j[e] < m.height - 1 ? m.pitch : 0));
