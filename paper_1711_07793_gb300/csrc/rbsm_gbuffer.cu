@@ -13,6 +13,7 @@
 #include "rbsm.h"
 #include "rbsm_device.cuh"
 #include "rbsm_host.h"
+#include "rbsm_rules.h"
 
 namespace rbsm {
 namespace {
@@ -65,6 +66,14 @@ gbuffer_kernel(const MapDev m, const GBufDev g, float *__restrict__ sil, float *
                uint16_t *__restrict__ codes, int max_dist, bool vec_planes)
 {
     constexpr int kWarps = kThreads / 32;
+    // a CTA owns every gridDim.x-th run of kRun tiles.  Short runs: where a shadow
+    // edge runs along the rows of fragments, all the fragments of several tiles
+    // in a row walk, and their walks, a line of the map per lane and step,
+    // are bound by the L1 of the SM they share (1414x1414 pixels whose rows run
+    // along the columns of a 2048^2 map, a straight edge along them, with a texture:
+    // 97 us with runs of 20, 41 with 5, 34 with 2; without the edge 17 / 19 / 19.
+    // 4 frames of 3840x2160: 193.7 / 194.4 / 196.1).
+    constexpr unsigned kRun = kThreads == kGbufferLargeThreads ? 5 : kWarps;
     __shared__ WarpQueue wq[kWarps];
     // the next job's kernel (launched as a programmatic dependent when the
     // jobs share no output) may take SMs as this one's CTAs finish
@@ -81,7 +90,7 @@ gbuffer_kernel(const MapDev m, const GBufDev g, float *__restrict__ sil, float *
     const long long n = (long long)g.width * g.height;
     const long long tiles = (n + kWarpTile - 1) / kWarpTile;
     auto tile_of = [&](unsigned k) {
-        return ((long long)(k / kWarps) * gridDim.x + blockIdx.x) * kWarps + k % kWarps;
+        return ((long long)(k / kRun) * gridDim.x + blockIdx.x) * kRun + k % kRun;
     };
     long long tile = tile_of((unsigned)warp);
     if (tile >= tiles)
@@ -198,22 +207,16 @@ gbuffer_kernel(const MapDev m, const GBufDev g, float *__restrict__ sil, float *
     drain(queued, true);
 }
 
-template <int MODE, bool CODES, int TEX>
+template <int MODE, bool CODES, int TEX, int kThreads>
 int launch_gbuffer(const MapDev &map, const GBufDev &g, float *sil, float *fil, uint16_t *codes, bool vec,
-                   int max_dist, bool overlap, cudaStream_t stream)
+                   int max_dist, bool overlap, int sms, cudaStream_t stream)
 {
-    // two CTAs of 20 warps per SM at 48 registers: 201 us for 4 frames of
-    // 3840x2160 pixels, against 213 with four of 8 warps at 64 registers
-    constexpr int kThreads = 640;
     auto kern = gbuffer_kernel<MODE, CODES, kThreads, TEX>;
     static KernelSetup setup;
     int occupancy = 0;
     int rc = setup.get(kern, kThreads, 0, &occupancy);
     if (rc != RBSM_OK)
         return rc;
-    const int sms = device_sm_count();
-    if (sms <= 0)
-        return cuda_fail(cudaErrorNoDevice);
     const long long n = (long long)g.width * g.height;
     const long long warp_tiles = (n + kWarpTile - 1) / kWarpTile;
     const long long blocks_needed = (warp_tiles + kThreads / 32 - 1) / (kThreads / 32);
@@ -250,8 +253,15 @@ template <int MODE, bool CODES>
 int launch_gbuffer(const MapDev &map, const GBufDev &g, float *sil, float *fil, uint16_t *codes, bool vec,
                    int max_dist, bool overlap, cudaStream_t stream)
 {
-    return map.tex ? launch_gbuffer<MODE, CODES, 1>(map, g, sil, fil, codes, vec, max_dist, overlap, stream)
-                   : launch_gbuffer<MODE, CODES, 0>(map, g, sil, fil, codes, vec, max_dist, overlap, stream);
+    const int sms = device_sm_count();
+    if (sms <= 0)
+        return cuda_fail(cudaErrorNoDevice);
+    constexpr int kLarge = kGbufferLargeThreads, kSmall = kGbufferSmallThreads;
+    if (gbuffer_large(g.width, g.height, sms))
+        return map.tex ? launch_gbuffer<MODE, CODES, 1, kLarge>(map, g, sil, fil, codes, vec, max_dist, overlap, sms, stream)
+                       : launch_gbuffer<MODE, CODES, 0, kLarge>(map, g, sil, fil, codes, vec, max_dist, overlap, sms, stream);
+    return map.tex ? launch_gbuffer<MODE, CODES, 1, kSmall>(map, g, sil, fil, codes, vec, max_dist, overlap, sms, stream)
+                   : launch_gbuffer<MODE, CODES, 0, kSmall>(map, g, sil, fil, codes, vec, max_dist, overlap, sms, stream);
 }
 
 struct Span {

@@ -51,4 +51,15 @@ inline bool light_spread_rows(int width, int height, int sms)
     return tiles > 32 && tiles <= 8LL * sms;
 }
 
+// Depth buffers: CTAs of 640 threads (two per SM) where there are 64 tiles of
+// 128 pixels for every SM, else of 256 (five per SM), both at 48 registers (us,
+// 640 / 256, both answers, with a texture: 320x240 14.0 / 12.1, 4 frames of 1280x720
+// 52.5 / 46.4, below the line; 1920x1080 29.2 / 29.4, silhouettes alone 24.9 /
+// 26.6, and one frame of 3840x2160 52.7 / 54.7, above).
+constexpr int kGbufferLargeThreads = 640, kGbufferSmallThreads = 256;
+inline bool gbuffer_large(int width, int height, int sms)
+{
+    return ((long long)width * height + 127) / 128 >= 64LL * sms;
+}
+
 }  // namespace rbsm

@@ -47,3 +47,10 @@ def test_light_pass_tiles(rule, size, rects, spheres, scale_in_range, large):
                                         (2048, 2048, False)])
 def test_light_pass_rows(rule, w, h, spread):
     assert rule("light_spread_rows(%d, %d, %d)" % (w, h, SMS)) == spread
+
+
+@pytest.mark.parametrize("w,h,large", [(320, 240, False), (1280, 720, False), (128, 64 * SMS - 1, False),
+                                       (127, 64 * SMS, False), (128, 64 * SMS, True), (1920, 1080, True),
+                                       (3840, 2160, True), (65536, 65536, True)])
+def test_depth_buffer_ctas(rule, w, h, large):
+    assert rule("gbuffer_large(%d, %d, %d)" % (w, h, SMS)) == large
