@@ -84,8 +84,8 @@ struct PlainJobs {
 };
 
 // Persistent warps over the warp tiles of one fragment set.  A CTA owns every
-// gridDim.x-th run of kRun consecutive tiles, so the tiles in flight gather
-// from one compact region of the shadow map, and its warps take them one at a
+// gridDim.x-th run of kRun consecutive tiles, so the tiles in flight on the GPU
+// gather from one compact region of the shadow map, and its warps take them one at a
 // time from a counter in shared memory: a tile along a shadow edge drains
 // several rounds of walks (4 us each) and holds up one warp while the others
 // take the tiles after it.  (A fixed share for each warp: 60.8 against 54.1 us
@@ -98,11 +98,17 @@ plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restric
              float *__restrict__ fil, uint16_t *__restrict__ codes, int max_dist, bool vec_planes)
 {
     constexpr int kWarps = kThreads / 32;
-    // runs of 16 tiles share the frame out more evenly than runs of a CTA's
-    // 32 (filtering 3840x2160 / 2560x1440, silhouette 1920x1080 / 1277x719
-    // unaligned: 51.5 / 33.2 / 19.8 / 20.6 us with 32, 49.2 / 31.8 / 20.2 /
-    // 18.9 with 16, 50.3 / 31.0 / 19.9 / 20.0 with 4)
-    constexpr unsigned kRun = kWarps < 16 ? kWarps : 16;
+    // runs of 2 tiles in the large CTAs.  Where a shadow edge runs along the rows
+    // of fragments, all the fragments of several tiles in a row walk, and their
+    // walks, a line of the map per lane and step, are bound by the L1 of
+    // the SM they share (1414x1414 fragments whose rows run along the columns of a
+    // 2048^2 map, a straight edge along them, filtering with a texture: 77.0 us with
+    // runs of 16, 41.7 with 4, 32.9 with 2; without the edge 17).  Elsewhere
+    // (filtering 3840x2160, silhouette 1920x1080, 1277x719 unaligned): 46.5 /
+    // 19.4 / 17.6 us with 16, 46.7 / 19.4 / 18.9 with 4, 46.4 / 19.8 / 18.4 with 2.
+    // The small CTAs keep a run for each round of their warps (320x240 11.4 us with
+    // runs of 8, 13.0 with 4).
+    constexpr unsigned kRun = kThreads == 1024 ? 2 : kWarps;
     __shared__ WarpQueue wq[kWarps];
     __shared__ float4 next[kWarps][3][32];
     __shared__ unsigned taken;                 // tiles of this CTA taken

@@ -17,7 +17,7 @@ from tests.test_gpu_shadowed_silhouettes import _time  # noqa: E402
 W, SIDE = 2048, 1414
 
 
-@pytest.mark.parametrize("what", ["depth buffer"])
+@pytest.mark.parametrize("what", ["depth buffer", "filter", "silhouette", "rpcf1"])
 def test_an_edge_along_the_rows(what):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -26,11 +26,18 @@ def test_an_edge_along_the_rows(what):
     from paper_1711_07793_gb300 import api
     depth = torch.full((W, W), 1.0, device="cuda")
     tex = api.MapTexture(depth)
-    m = np.zeros((4, 4), np.float32)
-    m[0, 1] = m[1, 0] = 1.0 / SIDE
-    m[2, 2] = m[3, 3] = 1.0
-    job = api.GBufferJob(tex, torch.full((SIDE, SIDE), 0.75, device="cuda"), m, mode=2)
-    call, vis = (lambda: api.rbsm_visibility_gbuffer([job], mode=2)), job.vis_filter
+    if what == "depth buffer":
+        m = np.zeros((4, 4), np.float32)
+        m[0, 1] = m[1, 0] = 1.0 / SIDE
+        m[2, 2] = m[3, 3] = 1.0
+        job = api.GBufferJob(tex, torch.full((SIDE, SIDE), 0.75, device="cuda"), m, mode=2)
+        call, vis = (lambda: api.rbsm_visibility_gbuffer([job], mode=2)), job.vis_filter
+    else:
+        t = (torch.arange(SIDE, device="cuda").float() + 0.5) / SIDE
+        xyz = t.repeat_interleave(SIDE), t.repeat(SIDE), torch.full((SIDE * SIDE,), 0.75, device="cuda")
+        vis = torch.empty_like(xyz[0])
+        call = {"filter": lambda: api.rsmss_filter(tex, *xyz, vis=vis), "rpcf1": lambda: api.rbsm_rpcf(tex, *xyz, k=1, vis=vis),
+                "silhouette": lambda: api.rbsm_visibility(tex, *xyz, vis=vis)}[what]
     plain = _time(call)
     assert bool((vis == 1).all())
     depth[:, :W // 2] = 0.1
