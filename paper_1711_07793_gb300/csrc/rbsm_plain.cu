@@ -91,8 +91,17 @@ struct PlainJobs {
 // take the tiles after it.  (A fixed share for each warp: 60.8 against 54.1 us
 // on 3840x2160 fragments, filtering, with CTAs of 8 warps.)  The next tile
 // waits in shared memory (cp.async), not in registers.
+//
+// Registers: 48 in the small CTAs, five to an SM, and 56 in the large ones, one to an
+// SM.  56 leave 8192 registers and 1024 threads of the SM to kernels on other
+// streams; the 63 that two of the large ones would take leave them nothing,
+// and they wait for the call to end: with 50 calls of filtering 3840x2160 on one
+// stream, 400 kernels over 4 MB on another are done after 2.77 ms with 63 and 1.43
+// with 56 (0.75 alone), and both streams after 2.78 and 2.52 ms.  Alone, filtering 3840x2160
+// / silhouette 1920x1080 / 1277x719 unaligned: 46.4 / 19.8 / 18.4 us with 63, 46.7 /
+// 20.2 / 17.9 with 56.
 template <int MODE, bool CODES, int kThreads, int TEX>
-__global__ void __launch_bounds__(kThreads, kThreads == 1024 ? 1 : 1280 / kThreads)
+__global__ void __launch_bounds__(kThreads) __maxnreg__(kThreads == 1024 ? 56 : 48)
 plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restrict__ y,
              const float *__restrict__ z, long long n, float *__restrict__ sil,
              float *__restrict__ fil, uint16_t *__restrict__ codes, int max_dist, bool vec_planes)
