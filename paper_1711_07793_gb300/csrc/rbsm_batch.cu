@@ -123,13 +123,23 @@ int uniform_mode(const BatchArgs &a)
 }
 
 // Whether a batch of one (mode, codes) pair takes the kernels for maps
-// without textures (UMODE + 6): no map it samples has one, and most of its
-// fragments sample maps of at least twice as many texels as the job has
-// fragments.  There single fragments 32 apart touch half the lines a pair
-// does (8 frames of 3840x2160 on 8192^2 maps 583 -> 495 us, one 91 -> 80);
-// fragments that share texels are served by either, and the pairs cost fewer
-// accesses to shared memory (64 cascade jobs, half of them on maps of fewer
-// texels than fragments: 417 us with pairs, 423 with single ones).
+// without textures (UMODE + 6): no map it samples has one, and three quarters
+// of its fragments sample maps of at least twice as many texels as the job has
+// fragments.  What decides is how far apart in the map neighbouring fragments
+// fall: single fragments 32 apart touch half the lines that pairs do where each
+// has a texel of its own, and with two answers to store the pairs cost
+// less where they share texels (8 M fragments on a 4096^2 map at a step of 0.1 /
+// 0.4 / 0.7 / 1.0 / 1.5 texels, both answers, pairs 42.1 / 54.5 / 63.4 / 75.5 / 86.9 us,
+// single ones 45.2 / 55.7 / 61.2 / 66.0 / 76.3; filtering alone 41.0 / 52.7 / 61.2 /
+// 72.7 / 83.8 and 41.2 / 52.0 / 57.4 / 62.5 / 72.3).  The host does not see the
+// step, and texels per fragment of the whole map stand for it: too many for a view of
+// a small part of a map, which loses the few per cent above.  With k of 8 jobs a
+// texel apart and the others a tenth of one, both answers, pairs take 146.6 /
+// 148.4 / 148.5 / 148.5 us at k = 1 / 3 / 5 / 6 and single ones 149.0 / 144.5 / 137.7 /
+// 133.6; but of 64 cascade jobs on maps of 2048^2 to 256^2 a quarter count as wide and
+// fall 0.2 to 0.4 texels apart, 474.6 and 494.9 (on 4096^2 to 512^2, half of them wide,
+// 423.6 and 424.2).  At three quarters none of these batches is slower than with
+// pairs.
 bool untextured(const BatchArgs &a)
 {
     long long all = 0, wide = 0;

@@ -372,12 +372,12 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) batch_kernel(const __gri
         fetch_tile<kTex == 0>(t, lane, buf, c);
         if (more) {
             if (nt < job_lo || nt >= job_hi) {
-                // mostly a few jobs on (the claims advance through the list)
                 if (nt < job_lo)
                     njob = find_job(a, nt);
+                // mostly a few jobs on (the claims advance through the list)
 #pragma unroll 1
-                    while (njob + 1 < a.n_jobs && a.jobs[njob + 1].tile_start <= nt)
-                        ++njob;
+                while (njob + 1 < a.n_jobs && a.jobs[njob + 1].tile_start <= nt)
+                    ++njob;
                 job_lo = a.jobs[njob].tile_start;
                 job_hi = njob + 1 < a.n_jobs ? a.jobs[njob + 1].tile_start : total;
                 tn = job_tile(a.jobs[njob], njob, nt);

@@ -175,10 +175,12 @@ plain_kernel(const MapDev m, const float *__restrict__ x, const float *__restric
 
 // CTAs of 1024 threads (one per SM: 32 warps share the tiles out) where the
 // tiles give every SM's 32 warps one, else of 256, which put a small launch on
-// more SMs.  3840x2160 filtering / 1920x1080 silhouette: 52.5 / 22.4 us with
-// 1024, 53.1 / 23.0 with two of 640, 52.2 / 24.4 with four of 320, 54.3 / 23.3
-// with five of 256 (before the walks' pairs of steps and the runs of 16:
-// 49.2 / 20.2; 47.2 / 19.8 with single fragments 32 apart).
+// more SMs.  Filtering 3840x2160 / silhouette 1920x1080 / 1277x719 unaligned: 47.4
+// / 20.5 / 18.1 us with 1024, 48.6 / 19.9 / 19.5 with two of 512, 51.7 / 23.8 / 20.4 with
+// two of 640, 53.3 / 23.4 / 19.9 with four of 320, 52.3 / 21.5 / 20.1 with five of 256.
+// Around the line (with a texture, silhouette / filtering, 256 and 1024): 640x480, 16
+// tiles per SM, 10.9 / 13.0 and 12.7 / 13.4; 960x540, 27, 13.0 / 14.1 and 12.4 / 14.1;
+// 1024x768, 40, 13.3 / 13.5 and 13.9 / 14.2; 1280x720, 47, 15.3 / 16.1 and 14.4 / 15.8.
 bool plain_large(int64_t n, int sms) { return (n + kWarpTile - 1) / kWarpTile >= 32LL * sms; }
 
 template <int MODE, bool CODES, int kThreads, int TEX>

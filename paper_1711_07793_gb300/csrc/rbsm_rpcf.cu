@@ -33,8 +33,12 @@ namespace {
 
 // One CTA of 32 warps per SM for k > 1 (two of 16 warps: 143.8 against 134.5
 // us at k = 3, four of 8: 159.7; the larger the CTA, the more strips its
-// warps share out), and for k = 1, whose kernel fits 48 registers, two of 20
-// (61.1 us with one of 32, 56.7 with these).  3840x2160 fragments.
+// warps share out; 3840x2160 fragments), and for k = 1, whose kernel fits 48
+// registers, two of 20: it gets calls of fewer than 32 tiles of 128 per SM
+// (rpcf_entry), where five of 8 and one of 32 come out about as well (320x240 /
+// 480x270 / 640x480 / 960x540 fragments, with a texture: 7.2 / 8.3 / 11.2 / 14.1 us with
+// two of 20, 7.2 / 7.6 / 11.7 / 14.7 with five of 8, 7.3 / 8.0 / 11.3 / 14.1 with one of
+// 32).
 template <int K>
 constexpr int kRpcfThreads = K == 1 ? 640 : 1024;
 
@@ -244,8 +248,8 @@ __device__ __forceinline__ void block_bits(const MapDev &m, float u, float v, fl
 // rounds of the longest walks.  A warp used to own a tile of 128 fragments
 // (up to 1152 samples, 36 rounds, at k = 3), and the tiles came from a fixed
 // partition or one at a time from a global counter; 3840x2160 fragments on
-// an 8192^2 map, k = 1 / 3 / 5: 66 / 179 / 488 us with tiles from the
-// counter, 56.8 / 128.7 / 288 us now.
+// an 8192^2 map, k = 3 / 5: 179 / 488 us with tiles from the counter, 128.7 /
+// 288 us now.
 constexpr unsigned kRun = 8;       // 16: 161.7 against 159.7 us, and 48 against 32.4 us for 320x240 fragments
 
 template <int K, int kThreads>
@@ -520,8 +524,9 @@ int rpcf_entry(const rbsm_map *map, const rbsm_frags *frags, float *vis, int32_t
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // k = 1 is rsmss_filter: with tiles enough for CTAs of 1024 its kernel
     // (3840x2160 / 1277x719 fragments 47.0 / 14.9 against 57.6 / 16.5 us here;
-    // 3840x2160 without a texture 66.6 against 75.8); on few fragments one strip
-    // per warp finishes sooner (one call on 320x240 22.3 against 25.7)
+    // 3840x2160 without a texture 66.6 against 75.8); on fewer fragments one
+    // strip per warp finishes sooner (320x240 / 640x480 / 960x540 7.2 / 11.2 / 14.1
+    // us here, 10.4 / 12.0 / 14.9 with its CTAs of 256)
     if (k == 1 && plain_large(frags->n, device_sm_count()))
         return plain_entry(RBSM_MODE_FILTER, map, frags, vis, nullptr, params, stream);
     switch (k) {
